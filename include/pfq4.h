@@ -122,7 +122,8 @@ typedef struct pf_solve_opts {
     int precision;         /* PF_FP64 or PF_MIXED */
     double inner_tol;      /* PF_MIXED: relative residual reduction of each inner FP32 solve
                               (<= 0: PF_DEFAULT_INNER_TOL) */
-    int chunk;             /* CG iterations per captured graph launch (0 = automatic) */
+    int chunk;             /* CG iterations per captured graph launch, or per launch of the kernel that
+                              keeps the CG state of small batches on the chip (0 = automatic) */
     int warm_start;        /* 1: start from the previous solution held by the handle */
     int tune_schedule;     /* 1: on the first such solve of the handle, run a few CG iterations
                               as timed launches and move the persistent kernel's tile ranges so
@@ -145,7 +146,8 @@ typedef struct pf_solve_info {
 
 typedef struct pf_timing {
     double cg_kernel_ms;         /* summed device time of the fused CG-iteration launches (CUDA events) */
-    long long cg_launches;       /* number of such launches */
+    long long cg_launches;       /* number of such launches; where the CG state stays on the chip (one launch
+                                    runs many iterations): the iterations of the longest variant */
     double residual_kernel_ms;   /* summed device time of the FP64 true-residual launches */
     long long residual_launches;
     double solve_ms;             /* device time of the whole solve, events on the call's stream */

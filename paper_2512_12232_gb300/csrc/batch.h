@@ -43,6 +43,21 @@ struct CgConfig {                  // persistent grid + schedule of one fused-CG
   int tune_rounds = 0;               // timing-driven re-balances done
 };
 
+// How a batch runs with its CG state on the chip (resident.cu), per precision.
+struct ResPlan {
+  bool made = false, ok = false;     // the plan was looked for; the batch fits
+  size_t smem = 0;                   // dynamic shared memory of a CTA
+  int grid = 0, n_items = 0, qs = 0; // CTAs, (variant, block) items, sums per block
+  long long pw_half = 0;             // words of one parity of d_pw
+  void *d_var = nullptr, *d_items = nullptr;
+  int* d_ctrl = nullptr;             // [1 + nv] ticket, started CTAs per variant
+  unsigned* d_epoch = nullptr;       // [nv] number of the last exchange
+  unsigned long long* d_pw = nullptr;   // [2][qs][blocks][2] exchanged partial sums
+  unsigned long long* d_bc = nullptr;   // broadcast alpha, beta, stop and body values
+  unsigned long long* d_pbm = nullptr;  // [blocks] bodies in each block
+  int* d_blist = nullptr;               // per variant and body: the blocks that hold its nodes
+};
+
 // One coarse level (l >= 1) of the geometric multigrid preconditioner, all variants packed:
 // variant v's level-l nodes (i, j) at off[v] + j (nx_l + 1) + i, each variant's block
 // starting on a multiple of 256 nodes (a 256-thread block never spans two variants).
@@ -121,6 +136,7 @@ struct Batch {
   bool cg_tune = false;              // re-balance the fused-CG schedule from timed launches
   int tuned_stages[2] = {2, 2};     // pipeline depth picked by the autotuner, per precision
   bool stages_tuned[2] = {false, false};
+  ResPlan res[2];                    // [precision]
   int nsm = 0;
   long long Rtot = 0;                // rows of the batch's 2-D node arrays (Vtot / P)
   int P = 0;                         // common row pitch
@@ -257,6 +273,11 @@ pf_status solve_core(Batch& b, double U, const pf_solve_opts& o, double* dev_psi
 long long* lbase_cached(Batch& b);
 void export_psi(Batch& b, double* dev_psi);
 void body_values(Batch& b, std::vector<double>& C);
+
+// resident.cu
+bool resident_ready(Batch& b, int precision);
+void launch_resident(Batch& b, int precision, int max_it);
+void drop_resident(Batch& b);
 
 // mg.cu
 void mg_setup(Batch& b);

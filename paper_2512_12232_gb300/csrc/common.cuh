@@ -52,6 +52,8 @@ constexpr uint8_t TILE_GEN64 = 1;     // a cell of the tile's window needs store
 constexpr uint8_t TILE_GEN32 = 2;     // ... stored FP32 K_e
 constexpr uint8_t TILE_PLAIN64 = 4;   // window all FREE, no TILE_GEN64 cell
 constexpr uint8_t TILE_PLAIN32 = 8;   // window all FREE, no TILE_GEN32 cell
+constexpr uint8_t TILE_ROW64 = 16;    // a FREE or BODY node of the tile whose four cells are not all active
+constexpr uint8_t TILE_ROW32 = 32;    // ones without stored FP64 (FP32) K_e
 
 // solver phases (per variant)
 constexpr int PH_CG = 0, PH_RESID = 1, PH_DONE = 2;

@@ -590,8 +590,11 @@ __global__ void k_stiffness(const DevVariant* var, const int* tile_var, const in
       if (cst != CUT_OK) {
         atomic_min_double(&dmin, -1.0);              // refused cell: the mesh is invalid
       } else if (cp.n == 0 && !disp) {
-        // an undisplaced hx-by-hy rectangle: every reader of stored K_e uses the
-        // closed-form constants for it, and det J = (hx/2)(hy/2) at every Gauss point
+        // an undisplaced hx-by-hy rectangle: det J = (hx/2)(hy/2) at every Gauss point.
+        // The closed-form constants are stored for the resident CG, which reads the
+        // coefficients of every cell around a node without looking at tags (inactive cells
+        // and those outside the grid hold zeros); every other reader takes the constants
+        for (int m = 0; m < 6; ++m) K64[m * Vtot + n] = V.kr64[m];
         atomic_min_double(&dmin, 0.25 * V.hx * V.hy);
       } else {
         double k6[6], dm;
@@ -632,14 +635,15 @@ __global__ void k_stiffness(const DevVariant* var, const int* tile_var, const in
 //     FP32): every node of its window i0-1 .. i0+CTX, j0-1 .. j0+CTY exists and is FREE
 //     (so every cell is active) and no cell needs stored coefficients, which lets the
 //     fused CG step skip the tags; and how many of its nodes carry an operator row
-//     (FREE or BODY)?  The counts feed the cost estimate of the fused-CG schedule.
+//     (FREE or BODY)?  Bits 4 and 5: some such node's row needs more than the rectangle
+//     constants (a stored, inactive or missing cell around it).  The counts feed the cost estimate of the fused-CG schedule.
 __global__ void k_tile_general(const DevVariant* var, const int* tile_var, const int2* tile_ij, const uint8_t* tag,
                                uint8_t* gen, int* act) {
   __shared__ int sh[NT / 32 + 1];
   const long long t = blockIdx.x;
   const DevVariant& V = var[tile_var[t]];
   const int2 ij = tile_ij[t];
-  int g64 = 0, g32 = 0, na = 0, allfree = 1;
+  int g64 = 0, g32 = 0, na = 0, allfree = 1, r64 = 0, r32 = 0;
   for (int q = linear_tid(); q < (CTX + 1) * (CTY + 1); q += NT) {
     const int i = ij.x - 1 + q % (CTX + 1), j = ij.y - 1 + q / (CTX + 1);
     if (i >= 0 && j >= 0 && i < V.nx && j < V.ny) {
@@ -651,8 +655,20 @@ __global__ void k_tile_general(const DevVariant* var, const int* tile_var, const
   for (int q = linear_tid(); q < CTX * CTY; q += NT) {
     const int i = ij.x + q % CTX, j = ij.y + q / CTX;
     if (i <= V.nx && j <= V.ny) {
-      const int k = tag[V.base + (long long)j * V.P + i] & KIND_MASK;
-      na += (k == K_FREE || k == K_BODY);
+      const long long n = V.base + (long long)j * V.P + i;
+      const int k = tag[n] & KIND_MASK;
+      const bool has_row = k == K_FREE || k == K_BODY;
+      na += has_row;
+      if (has_row) {
+        if (i == 0 || j == 0 || i == V.nx || j == V.ny) {
+          r64 = r32 = 1;
+        } else {
+          const uint8_t all = tag[n] & tag[n - 1] & tag[n - V.P] & tag[n - V.P - 1];
+          const uint8_t any = tag[n] | tag[n - 1] | tag[n - V.P] | tag[n - V.P - 1];
+          r64 |= !(all & CELL_ACTIVE) || (any & CELL_GENERAL);
+          r32 |= !(all & CELL_ACTIVE) || (any & CELL_GEN32);
+        }
+      }
     }
   }
   for (int q = linear_tid(); q < (CTX + 2) * (CTY + 2); q += NT) {
@@ -663,11 +679,13 @@ __global__ void k_tile_general(const DevVariant* var, const int* tile_var, const
   g64 = __syncthreads_or(g64);
   g32 = __syncthreads_or(g32);
   allfree = __syncthreads_and(allfree);
+  r64 = __syncthreads_or(r64);
+  r32 = __syncthreads_or(r32);
   int tot;
   block_exscan(na, &tot, sh);
   if (linear_tid() == 0) {
     gen[t] = (uint8_t)((g64 ? TILE_GEN64 : 0) | (g32 ? TILE_GEN32 : 0) | (allfree && !g64 ? TILE_PLAIN64 : 0) |
-                       (allfree && !g32 ? TILE_PLAIN32 : 0));
+                       (allfree && !g32 ? TILE_PLAIN32 : 0) | (r64 ? TILE_ROW64 : 0) | (r32 ? TILE_ROW32 : 0));
     act[t] = tot;
   }
 }
@@ -1208,6 +1226,7 @@ void set_coords(Batch& b, int v, const double* dev_xy) {
   refresh_apply_groups(b);   // the stand-alone operator's plain-tile bits follow the tile flags
   destroy_phi_view(b);       // its tile flags were made from the old coordinates
   destroy_mg(b);             // and the multigrid operators from the old element matrices
+  drop_resident(b);          // the resident CG's blocks follow the tile flags
   b.solved = false;          // any earlier solution belongs to the old coordinates
 }
 

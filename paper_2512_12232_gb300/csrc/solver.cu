@@ -1822,6 +1822,10 @@ static cudaGraphExec_t get_graph(Batch& b, int precision, int chunk) {
   return ex;
 }
 
+// Iterations of one launch of the resident CG at most: a launch that is not done by then
+// saves its state and the next one goes on (about 0.3 s at 5 us an iteration).
+constexpr int RESIDENT_ITERS = 1 << 16;
+
 // Iterations per captured graph of the preconditioned CG (each about 40 kernels).
 constexpr int PCG_CHUNK = 4;
 
@@ -1969,7 +1973,8 @@ pf_status solve_core(Batch& b, double U, const pf_solve_opts& o, double* dev_psi
     if (hdone[1]) throw Error{PF_ETIMEOUT, "a bounded wait in the CG kernel gave up (TMA tile not delivered)"};
     return (double)ms / n;
   };
-  const bool tune = b.cg_tune && o.k_max > 0 && !getenv("PFQ4_CG_STAGES") && !pcg;
+  const bool resident = !pcg && o.k_max > 0 && resident_ready(b, prec);
+  const bool tune = b.cg_tune && o.k_max > 0 && !getenv("PFQ4_CG_STAGES") && !pcg && !resident;
   if (tune && !b.stages_tuned[prec]) {
     double best = 1e300;
     int best_ns = b.cg_stages;
@@ -1985,14 +1990,15 @@ pf_status solve_core(Batch& b, double U, const pf_solve_opts& o, double* dev_psi
     b.tuned_stages[prec] = best_ns;
     b.stages_tuned[prec] = true;
   }
-  cudaGraphExec_t ex = pcg ? get_pcg_graph(b, chunk) : get_graph(b, prec, chunk);
-  CgConfig& cc = cg_config(b, prec, b.cg_stages);
-  if (!pcg &&
+  cudaGraphExec_t ex = resident ? nullptr : pcg ? get_pcg_graph(b, chunk) : get_graph(b, prec, chunk);
+  CgConfig none;
+  CgConfig& cc = resident ? none : cg_config(b, prec, b.cg_stages);
+  if (!pcg && !resident &&
       (cc.active.size() != (size_t)b.nv || std::find(cc.active.begin(), cc.active.end(), 0) != cc.active.end())) {
     cc.active.assign(b.nv, 1);                   // a solve starts with every variant running
     cg_sched_write(b, cc);
   }
-  if (!pcg && b.cg_tune && o.k_max > 0 && (long long)cc.tile_cost.size() >= 2LL * cc.G) {
+  if (!pcg && !resident && b.cg_tune && o.k_max > 0 && (long long)cc.tile_cost.size() >= 2LL * cc.G) {
     const int rounds = env_int("PFQ4_CG_TUNE_ROUNDS", CG_TUNE_ROUNDS, 0, 16);
     const int per_round = env_int("PFQ4_CG_TUNE_LAUNCHES", CG_TUNE_LAUNCHES, 1, 16);
     for (; cc.tune_rounds < rounds; ++cc.tune_rounds) {
@@ -2004,6 +2010,7 @@ pf_status solve_core(Batch& b, double U, const pf_solve_opts& o, double* dev_psi
     }
   }
   // k_max == 0 (internal use): only the initial residual, which measures ||b||
+  if (resident) chunk = o.chunk > 0 ? o.chunk : RESIDENT_ITERS;
   const long long max_chunks = o.k_max == 0 ? 0 : o.k_max / chunk + 1000;
   // Chunks are queued two ahead of the host: slot k holds events (start, after the CG
   // graph, after the refinement kernels) and the pinned poll words / variant states
@@ -2019,7 +2026,8 @@ pf_status solve_core(Batch& b, double U, const pf_solve_opts& o, double* dev_psi
   auto issue = [&](long long c) {
     const int k = (int)(c % SLOTS);
     PF_CUDA(cudaEventRecord(b.ev[6 + 3 * k], s));
-    PF_CUDA(cudaGraphLaunch(ex, s));
+    if (resident) launch_resident(b, prec, chunk);
+    else PF_CUDA(cudaGraphLaunch(ex, s));
     PF_CUDA(cudaEventRecord(b.ev[7 + 3 * k], s));
     launch_resid_only(b, prec, s);
     PF_CUDA(cudaMemcpyAsync(hdone + 2 * k, b.n_done, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -2035,14 +2043,14 @@ pf_status solve_core(Batch& b, double U, const pf_solve_opts& o, double* dev_psi
     PF_CUDA(cudaEventElapsedTime(&ms2, b.ev[7 + 3 * k], b.ev[8 + 3 * k]));
     cg_ms += ms1;
     res_ms += ms2;
-    launches += chunk;
+    if (!resident) launches += chunk;
     rlaunches += 1;
     if (hdone[2 * k + 1]) throw Error{PF_ETIMEOUT, "a bounded wait in the CG kernel gave up (TMA tile not delivered)"};
     if (hdone[2 * k] >= b.nv) {
       finished = true;
       return;
     }
-    if (pcg) return;                             // its kernels take every variant's tiles each launch
+    if (pcg || resident) return;                 // the preconditioned kernels take every variant's tiles each launch
     // spread the grid over the variants still running once enough work has finished
     std::vector<char> act(b.nv);
     for (int v = 0; v < b.nv; ++v) act[v] = b.h_vs[(size_t)k * b.nv + v].phase != PH_DONE;
@@ -2071,9 +2079,9 @@ pf_status solve_core(Batch& b, double U, const pf_solve_opts& o, double* dev_psi
   PF_CUDA(cudaEventRecord(b.ev[4], s));
   // kernels launched: k_init, slot seeding, the tuning launches and every queued chunk
   // (CG graph + fold + residual), no-op chunks after the last variant finished included
-  const long long tuned_launches = launches - (long long)(rlaunches - 1) * chunk;
-  b.launches += 1 + (n_slots > 0 ? 1 : 0) + tuned_launches + issued * chunk * (pcg ? pcg_launches_per_iter(b) : 1) +
-                (1 + issued) * 2;
+  const long long tuned_launches = resident ? 0 : launches - (long long)(rlaunches - 1) * chunk;
+  b.launches += 1 + (n_slots > 0 ? 1 : 0) + tuned_launches +
+                (resident ? issued : issued * chunk * (pcg ? pcg_launches_per_iter(b) : 1)) + (1 + issued) * 2;
   std::vector<VarState> fin(b.nv);
   PF_CUDA(cudaMemcpyAsync(fin.data(), b.state, b.nv * sizeof(VarState), cudaMemcpyDeviceToHost, s));
   PF_CUDA(cudaStreamSynchronize(s));
@@ -2097,6 +2105,7 @@ pf_status solve_core(Batch& b, double U, const pf_solve_opts& o, double* dev_psi
     const long long n_gen = prec == PF_MIXED ? b.hv[v].n_gen32_cells : M.n_general_cells;
     const double bv = per_node_free * M.n_free + per_body * M.n_body_nodes + 1.0 * M.n_nodes + per_gen * n_gen;
     if (!pcg) bytes_done += bv * (double)S.iters;
+    if (resident) launches = std::max(launches, S.iters);   // a resident iteration counts as a launch of the streaming kernel
     if (info) {
       info[v].iters = S.iters;
       info[v].refinements = std::max(0, S.n_resid - 1);

@@ -1,0 +1,87 @@
+"""The CG with its state on the chip (csrc/resident.cu) against the oracle's direct solves, at
+the sizes where its block cut can go wrong: grids of a few nodes, one block, blocks with a
+ragged last row and column, half strips of two rows, wide and tall grids, bodies that share a
+thread's strip, natural sides (rows without all four cells), batches that queue, and a solve
+cut into many launches.  Tolerances are those of the GPU parity tests: at a true residual tol
+the error of psi is tol times a condition number of up to 1e5 on these grids, so 1e-10 in
+relative L2 for FP64 at 1e-15 x 1e5; 1e-6 in mixed precision at 1e-12."""
+import functools
+
+import numpy as np
+import pytest
+
+from oracle import mesh as OM, solve as OS, system as OSY
+from paper_2512_12232_gb300 import workloads as W
+from tests.gpu_util import rel_l2
+
+pytestmark = pytest.mark.gpu
+
+D, N = W.BC_DIRICHLET_UY, W.BC_NATURAL
+
+
+def _case(nx, ny, bodies, sweeps=8, bc=(D, D, D, D), box=(-4.0, 4.0, -2.0, 2.0)):
+    return W.Case(*box, nx, ny, np.asarray(bodies, dtype=np.float64).reshape(-1, 3), sweeps, bc)
+
+
+ONE = [[0.13, 0.07, 0.6]]
+CASES = {
+    "3x3_nodes": [_case(2, 2, [])],
+    "one_column_of_cells": [_case(33, 2, [])],
+    "one_block": [_case(40, 20, ONE)],
+    "ragged": [_case(101, 67, ONE)],
+    "wide": [_case(603, 37, [[0.13, 0.07, 0.9]])],
+    "tall": [_case(31, 301, ONE, box=(-2.0, 2.0, -4.0, 4.0))],
+    "natural": [_case(150, 75, ONE, bc=(N, N, D, D))],
+    "natural_three_sides": [_case(90, 45, ONE, bc=(D, N, N, N))],
+    "close_bodies": [_case(160, 80, [[-0.9, -0.62, 0.5], [-0.87, 0.55, 0.5], [0.6, 0.1, 0.4], [1.9, 0.0, 0.3]])],
+    "uneven_batch": [_case(64, 32, ONE), _case(200, 33, ONE), _case(48, 96, ONE, box=(-2.0, 2.0, -4.0, 4.0)),
+                     _case(97, 49, [])],
+    "queue": [_case(320 + 2 * k, 160 + k, [[0.13 + 0.001 * k, 0.07, 0.6]], 40) for k in range(20)],
+}
+
+
+@functools.lru_cache(maxsize=64)
+def _reference(name, v):
+    c = CASES[name][v]
+    m = OM.build_mesh(c.grid, c.bodies, c.sweeps, c.bc)
+    s = OSY.assemble(m, 1.0)
+    u, psi = OS.solve_direct(s)
+    return psi, u[s.n_free:]
+
+
+@pytest.fixture(scope="module")
+def api():
+    from paper_2512_12232_gb300 import api
+    return api
+
+
+@pytest.mark.parametrize("prec,tol,bound", [("fp64", 1e-13, 1e-10), ("mixed", 1e-12, 1e-6)])
+@pytest.mark.parametrize("name", list(CASES))
+def test_resident_solve_matches_oracle(api, name, prec, tol, bound):
+    cases = CASES[name]
+    p = api.PF_FP64 if prec == "fp64" else api.PF_MIXED
+    with api.batch_build(cases) as g:
+        for chunk in (0, 7):               # 7: every launch pauses and the next one goes on
+            if chunk and name in ("queue", "wide"):
+                continue
+            res = api.psi_solve(g, U=1.0, tol=tol, precision=p, chunk=chunk)
+            psi = res.psi.cpu().numpy()
+            for v in range(len(cases)):
+                if name == "queue" and v % 7:
+                    continue
+                ref, C = _reference(name, v)
+                assert res.info[v]["status"] == 0 and res.info[v]["rel_true_residual"] <= tol
+                assert rel_l2(psi[g.node_offsets[v]:g.node_offsets[v + 1]], ref) <= bound, (name, v, chunk)
+                k = g.body_offsets[v]
+                np.testing.assert_allclose(res.body_psi[k:k + len(C)], C, rtol=0, atol=10 * bound)
+        again = api.psi_solve(g, U=1.0, tol=tol, precision=p, chunk=chunk if name not in ("queue", "wide") else 0)
+    assert np.array_equal(again.psi.cpu().numpy(), psi)   # sums are taken in a fixed order
+
+
+def test_resident_iteration_cap(api):
+    """k_max ends a solve inside a launch with the capped status and a finite iterate."""
+    c = CASES["ragged"][0]
+    with api.mesh_build(c.grid, c.bodies, c.sweeps, c.bc) as g:
+        res = api.psi_solve(g, U=1.0, tol=1e-12, precision=api.PF_MIXED, k_max=11, raise_on_failure=False)
+        assert res.info[0]["iters"] == 11 and res.info[0]["status"] == 3   # PF_ENOT_CONVERGED
+        assert np.all(np.isfinite(res.psi.cpu().numpy()))
