@@ -953,7 +953,7 @@ __global__ void __launch_bounds__(RNT, 2) k_cg_resident(ResArgs<T> g) {
         const int parts = sh.parts;
         u64* const mine = sh.pw_var + (ep & 1) * g.pw_half + (long long)part * 2;
         if (warp == 0) {
-          double s = s_red[lane & 7][lane >> 3];
+          double s = (lane & 7) < RWARPS ? s_red[lane & 7][lane >> 3] : 0.0;
 #pragma unroll
           for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
           if ((lane & 7) == 0 && !drop) put_double(mine + (long long)(lane >> 3) * parts * 2, s, ep);

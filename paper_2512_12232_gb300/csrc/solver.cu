@@ -1246,6 +1246,129 @@ __global__ void __launch_bounds__(NT) k_body_sums(MeshDev m, const T* y, double*
   if (linear_tid() == 0) out[blockIdx.x] = s;
 }
 
+// y = A p straight from and to the caller's logical vectors, one 64 x 16 tile per CTA: p with a
+// one-node halo is converted to T into shared memory, each thread forms a vertical strip of
+// four rows, the result is widened on its way out.  Plain tiles (flags of k_tile_general) read
+// no tags and no coefficients.  Rows are formed by the functions of k_apply, with the same
+// bits, except FP64 plain tiles, which share the second differences between a strip's rows
+// (10.75 instead of 16 FP64 operations per node: the FP64 pipe is their bound).
+// Bytes per node: 8 read, 8 written (plus tags and coefficients off the plain tiles); the three
+// passes it replaces (copy to the padded vector, k_apply, copy back) moved 40 and a memset.
+template <typename T>
+__global__ void __launch_bounds__(NT, 4) k_apply_direct(MeshDev m, const int2* __restrict__ tij, const int* __restrict__ tvar,
+                                                     const uint8_t* __restrict__ tfl, const long long* __restrict__ lbase,
+                                                     const double* __restrict__ p, double* __restrict__ y) {
+  constexpr int FW = CTX + 2, FH = CTY + 2;
+  __shared__ T ps[FH][FW];
+  __shared__ uint8_t ts[FH][FW];
+  const int t = blockIdx.x, v = tvar[t];
+  const DevVariant& V = m.var[v];
+  const int nx = V.nx, ny = V.ny, P = V.P;
+  const long long row = nx + 1, lb = lbase[v];
+  const int2 ij = tij[t];
+  const int tid = linear_tid(), col = tid % CTX, r0 = (tid / CTX) * STRIP, i = ij.x + col;
+  const bool plain = (tfl[t] & (sizeof(T) == 4 ? TILE_PLAIN32 : TILE_PLAIN64)) != 0;
+  // this thread's halo position
+  int li = 0, lj = 0;
+  const bool halo = tid < 2 * FW + 2 * CTY;
+  if (tid < FW) li = tid;
+  else if (tid < 2 * FW) { li = tid - FW; lj = CTY + 1; }
+  else if (tid < 2 * FW + CTY) lj = 1 + tid - 2 * FW;
+  else { li = CTX + 1; lj = 1 + tid - 2 * FW - CTY; }
+  const int hi = ij.x - 1 + li, hj = ij.y - 1 + lj;
+  const double* const pc = p + lb + (ij.y + r0) * row + i;
+  double* const yc = y + lb + (ij.y + r0) * row + i;
+  if (plain) {                               // the whole window lies inside the grid
+    double c[STRIP], h = 0.0;
+#pragma unroll
+    for (int u = 0; u < STRIP; ++u) c[u] = pc[u * row];
+    if (halo) h = p[lb + hj * row + hi];
+#pragma unroll
+    for (int u = 0; u < STRIP; ++u) ps[1 + r0 + u][1 + col] = (T)c[u];
+    if (halo) ps[lj][li] = (T)h;
+    __syncthreads();
+    T win[STRIP + 2][3];
+#pragma unroll
+    for (int r = 0; r < STRIP + 2; ++r)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) win[r][k] = ps[r0 + r][col + k];
+    T kr[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) kr[k] = krect<T>(V)[k];
+    if (sizeof(T) == 8) {
+      T S[STRIP + 2];
+#pragma unroll
+      for (int r = 0; r < STRIP + 2; ++r) S[r] = (win[r][0] - win[r][1]) + (win[r][2] - win[r][1]);
+      const T c1 = T(2) * kr[0], c2 = T(2) * (kr[1] + kr[2]);
+      T dm = win[1][1] - win[0][1];
+#pragma unroll
+      for (int u = 0; u < STRIP; ++u) {
+        const T dp = win[u + 2][1] - win[u + 1][1];
+        yc[u * row] = fma(kr[1], S[u] + S[u + 2], fma(c2, dp - dm, c1 * S[u + 1]));
+        dm = dp;
+      }
+    } else {
+#pragma unroll
+      for (int u = 0; u < STRIP; ++u) {
+        const T nbh[3][3] = {{win[u][0], win[u][1], win[u][2]},
+                             {win[u + 1][0], win[u + 1][1], win[u + 1][2]},
+                             {win[u + 2][0], win[u + 2][1], win[u + 2][2]}};
+        yc[u * row] = (double)q4_row_rect<T>(nbh, kr);
+      }
+    }
+    return;
+  }
+  const long long n0 = V.base + (long long)(ij.y + r0) * P + i;
+#pragma unroll
+  for (int u = 0; u < STRIP; ++u) {
+    const bool in = i <= nx && ij.y + r0 + u <= ny;
+    ps[1 + r0 + u][1 + col] = in ? (T)pc[u * row] : T(0);
+    ts[1 + r0 + u][1 + col] = in ? m.tag[n0 + (long long)u * P] : K_INACT;
+  }
+  if (halo) {
+    const bool in = hi >= 0 && hj >= 0 && hi <= nx && hj <= ny;
+    ps[lj][li] = in ? (T)p[lb + hj * row + hi] : T(0);
+    ts[lj][li] = in ? m.tag[V.base + (long long)hj * P + hi] : K_INACT;
+  }
+  __syncthreads();
+  if (i > nx) return;
+  T kr[6];
+#pragma unroll
+  for (int k = 0; k < 6; ++k) kr[k] = krect<T>(V)[k];
+#pragma unroll
+  for (int u = 0; u < STRIP; ++u) {
+    if (ij.y + r0 + u > ny) break;
+    const int a = 1 + r0 + u, b = 1 + col;   // the node in the shared tile
+    T out = T(0);
+    const int kind = ts[a][b] & KIND_MASK;
+    if (kind == K_FREE || kind == K_BODY) {
+      const T nbh[3][3] = {{ps[a - 1][b - 1], ps[a - 1][b], ps[a - 1][b + 1]},
+                           {ps[a][b - 1], ps[a][b], ps[a][b + 1]},
+                           {ps[a + 1][b - 1], ps[a + 1][b], ps[a + 1][b + 1]}};
+      out = q4_row_nb<T, false, true>(nbh, ts[a][b], ts[a][b - 1], ts[a - 1][b - 1], ts[a - 1][b], nullptr, 0, 0,
+                                      n0 + (long long)u * P, P, kplane<T>(m), m.Vtot, kr);
+    }
+    yc[u * row] = (double)out;
+  }
+}
+
+// collapsed body rows of a logical vector: one CTA per global body, in k_body_sums' order
+__global__ void __launch_bounds__(NT) k_body_sums_logical(MeshDev m, const int* body_var, const long long* lbase,
+                                                          const double* y, double* out) {
+  __shared__ double scratch[NT / 32 + 1];
+  const int gb = blockIdx.x, v = body_var[gb];
+  const DevVariant& V = m.var[v];
+  const long long lb = lbase[v];
+  double s = 0.0;
+  const int e1 = m.body_ptr[gb + 1];
+  for (int e = m.body_ptr[gb] + linear_tid(); e < e1; e += NT) {
+    const unsigned rem = (unsigned)(m.body_nodes[e] - V.base);
+    s += y[lb + (long long)(rem / (unsigned)V.P) * (V.nx + 1) + rem % (unsigned)V.P];
+  }
+  s = block_sum(s, scratch);
+  if (linear_tid() == 0) out[gb] = s;
+}
+
 // ---------------------------------------------------------------- host side
 static MeshDev mesh_dev(const Batch& b) {
   MeshDev m;
@@ -1681,12 +1804,35 @@ void apply_timing(Batch& b, int precision, int reps, double* us, double* bytes) 
   if (bytes) *bytes = by;
 }
 
+// Input and output apart (the usual call): one kernel straight on the caller's vectors.  Where
+// they overlap, through the padded vectors: a tile must not see its neighbours' results.
+// Measured per call (GB300, with the Python binding), padded -> direct: 8193x4097 nodes, FP32,
+// 510 -> 222 us; 404x202 nodes, FP64, 95 -> 55 us.
 void apply_operator(Batch& b, int precision, const double* dev_p, double* dev_y, double* body_sums) {
-  ensure_apply_buffers(b);
   long long* lb = lbase_cached(b);
   const MeshDev m = mesh_dev(b);
-  const dim3 g2(512, b.nv);
   double* sums = body_sum_scratch(b);
+  long long total = 0;
+  for (const HostVariant& H : b.hv) total += H.stats.n_nodes;
+  const uintptr_t p0 = (uintptr_t)dev_p, y0 = (uintptr_t)dev_y, bytes = (uintptr_t)total * sizeof(double);
+  if (p0 + bytes <= y0 || y0 + bytes <= p0) {
+    const dim3 blk(TX, TY);
+    if (precision == PF_FP64)
+      k_apply_direct<double><<<(unsigned)b.Tcg, blk, 0, b.stream>>>(m, b.tile_cg_ij, b.tile_cg_var, b.tile_cg_gen, lb,
+                                                                    dev_p, dev_y);
+    else
+      k_apply_direct<float><<<(unsigned)b.Tcg, blk, 0, b.stream>>>(m, b.tile_cg_ij, b.tile_cg_var, b.tile_cg_gen, lb,
+                                                                   dev_p, dev_y);
+    if (b.B && body_sums) {
+      k_body_sums_logical<<<b.B, blk, 0, b.stream>>>(m, b.d_body_var, lb, dev_y, sums);
+      PF_CUDA(cudaMemcpyAsync(body_sums, sums, b.B * sizeof(double), cudaMemcpyDeviceToHost, b.stream));
+    }
+    PF_CUDA(cudaGetLastError());
+    PF_CUDA(cudaStreamSynchronize(b.stream));
+    return;
+  }
+  ensure_apply_buffers(b);
+  const dim3 g2(512, b.nv);
   if (precision == PF_FP64) {
     k_to_padded<double><<<g2, 256, 0, b.stream>>>(b.d_var, lb, dev_p, b.ap64[0]);
     PF_CUDA(cudaMemsetAsync(b.ap64[1], 0, b.Vtot * sizeof(double), b.stream));
