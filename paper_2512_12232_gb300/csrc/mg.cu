@@ -161,13 +161,15 @@ __device__ __forceinline__ bool lv_node(const long long* off, const int2* dims, 
   const long long o = off[v];
   if (o < 0) return false;
   const int2 d = dims[v];
-  const long long loc = (long long)blockIdx.x * blockDim.x + threadIdx.x - o;
-  if (loc >= (long long)(d.x + 1) * (d.y + 1)) return false;
+  // (one variant's level has fewer than 2^31 nodes: a 64-bit division here cost more than
+  // the sweep itself)
+  const unsigned loc = (unsigned)((long long)blockIdx.x * blockDim.x + threadIdx.x - o), w = (unsigned)d.x + 1u;
+  if (loc >= w * ((unsigned)d.y + 1u)) return false;
   q.v = v;
   q.nx = d.x;
   q.ny = d.y;
-  q.i = (int)(loc % (d.x + 1));
-  q.j = (int)(loc / (d.x + 1));
+  q.j = (int)(loc / w);
+  q.i = (int)(loc - (unsigned)q.j * w);
   q.k = o + loc;
   return true;
 }
@@ -316,6 +318,7 @@ struct FineArgs {
   MeshDev m;
   const int* tile_var;       // fused-CG tile list (64 x 16)
   const int2* tile_ij;
+  const uint8_t* tile_gen;   // its flags (TILE_PLAIN32: no tags, no coefficients needed)
   const VarState* st;
   const float* dinv0;
   float *x, *r, *z, *t, *res, *q;
@@ -417,6 +420,80 @@ __device__ __forceinline__ void block_dot_acc(Acc<float>& acc, double* part, dou
   }
 }
 
+// ---- plain tiles: every node of the tile and its halo is FREE and every cell an undisplaced
+// rectangle.  No tags, no bounds, no coefficients and no shared memory: a thread loads its
+// column's six rows (the strip and one above and below), takes the columns to either side from
+// its neighbour lanes (the warp's first and last lane load theirs), and all loads are in flight
+// before the first is used.  The operator row, the interpolation and the dot products are
+// formed in the order of the general tiles' code, so a value does not depend on which of the
+// two made it.  The general code spends most of its time on tags, bounds and 64-bit indices: per
+// launch on the 256-variant sweep (62.5 M nodes, 60 % of the tiles plain) the residual took 478 ->
+// 292 us, the post-smoothing with the prolongation 727 -> 521 us, the operator 479 -> 405 us, the
+// update 326 -> 290 us; on one 8192x4096 grid a whole solve took 126 -> 91 ms.
+struct PlainCols {
+  float c[FS + 2], e[FS + 2];   // the thread's column; the column outside the warp (lanes 0 and 31)
+};
+__device__ __forceinline__ void plain_load(PlainCols& q, const float* f, long long n0, int P, int lane) {
+  const float* p = f + n0 - P;
+  const int side = lane == 0 ? -1 : 1;
+#pragma unroll
+  for (int r = 0; r < FS + 2; ++r) {
+    q.c[r] = p[(long long)r * P];
+    q.e[r] = (lane == 0 || lane == 31) ? p[(long long)r * P + side] : 0.0f;
+  }
+}
+__device__ __forceinline__ void plain_apply(const PlainCols& q, const float* kr, int lane, float (&y)[FS]) {
+  float L[FS + 2], R[FS + 2];
+#pragma unroll
+  for (int r = 0; r < FS + 2; ++r) {
+    const float l = __shfl_up_sync(0xffffffffu, q.c[r], 1), u = __shfl_down_sync(0xffffffffu, q.c[r], 1);
+    L[r] = lane == 0 ? q.e[r] : l;
+    R[r] = lane == 31 ? q.e[r] : u;
+  }
+  const float k01 = kr[0], k02 = kr[1], k03 = kr[2], k12 = kr[3], k13 = kr[4], k23 = kr[5];
+#pragma unroll
+  for (int u = 0; u < FS; ++u) {
+    const float pc = q.c[u + 1];
+    const float dE = R[u + 1] - pc, dW = L[u + 1] - pc, dN = q.c[u + 2] - pc, dS = q.c[u] - pc;
+    const float dNE = R[u + 2] - pc, dNW = L[u + 2] - pc, dSE = R[u] - pc, dSW = L[u] - pc;
+    // (the roundings the compiler gives q4_row's sums, written out)
+    float s = fmaf(k03, dN, fmaf(k01, dE, __fmul_rn(k02, dNE)));
+    s = __fadd_rn(s, fmaf(k13, dNW, fmaf(k01, dW, __fmul_rn(k12, dN))));
+    s = __fadd_rn(s, fmaf(k23, dW, fmaf(k02, dSW, __fmul_rn(k12, dS))));
+    s = __fadd_rn(s, fmaf(k23, dE, fmaf(k03, dS, __fmul_rn(k13, dSE))));
+    y[u] = s;
+  }
+}
+// P e on rows j0 - 1 .. j0 + FS of fine column i (j0 a multiple of 4): along both axes an even
+// fine index takes its coarse node, an odd one half of each of its two.  (Odd last lines, which
+// copy their coarse node, are not on tiles that take this path.)
+__device__ __forceinline__ void plain_prolong(const float* cz, int w, int i, int j0, float (&e)[FS + 2]) {
+  const float* p = cz + (long long)(j0 / 2 - 1) * w;
+  const int ia = i >> 1, ib = (i + 1) >> 1;
+  const float wa = (i & 1) ? 0.5f : 1.0f, wb = (i & 1) ? 0.5f : 0.0f;
+  float A[FS / 2 + 2], B[FS / 2 + 2];
+#pragma unroll
+  for (int J = 0; J < FS / 2 + 2; ++J) {
+    A[J] = p[(long long)J * w + ia];
+    B[J] = p[(long long)J * w + ib];
+  }
+#pragma unroll
+  for (int r = 0; r < FS + 2; ++r) {
+    if (r & 1) {
+      const int J = (r + 1) / 2;
+      e[r] = fmaf(wb, B[J], wa * A[J]);
+    } else {
+      const int J = r / 2;
+      const float ha = 0.5f * wa, hb = 0.5f * wb;
+      e[r] = fmaf(hb, B[J + 1], fmaf(ha, A[J + 1], fmaf(hb, B[J], ha * A[J])));
+    }
+  }
+}
+__device__ __forceinline__ bool plain_tile(const FineArgs& a, const DevVariant& V, int2 ij, bool prolong) {
+  if (!(a.tile_gen[blockIdx.x] & TILE_PLAIN32)) return false;
+  return !prolong || (ij.x + CTX < V.nx && ij.y + CTY < V.ny);
+}
+
 // x += alpha p, r -= alpha q, z = dinv r (the first pre-smoothing sweep from zero, before
 // the forward body step's term, which k_mg_fwd subtracts next to the bodies); r.r.
 // Pointwise, FREE nodes only; a node is FREE exactly when its Jacobi factor is positive
@@ -434,8 +511,31 @@ __global__ void __launch_bounds__(NT) k_mg0_update(FineArgs a) {
   const float alpha = (float)S.alpha;
   const float* pc = a.p[S.buf];
   float rn[FS];
+  const bool plain = plain_tile(a, V, ij, false);
+  if (plain) {                         // one Jacobi factor for the whole tile
+    const long long n0 = V.base + (long long)(ij.y + r0) * V.P + i;
+    const float dn = a.dinv0[n0];
+    float pn[FS], xn[FS], qn[FS];
+#pragma unroll
+    for (int u = 0; u < FS; ++u) {
+      const long long n = n0 + (long long)u * V.P;
+      pn[u] = pc[n];
+      xn[u] = a.x[n];
+      rn[u] = a.r[n];
+      qn[u] = a.q[n];
+    }
+#pragma unroll
+    for (int u = 0; u < FS; ++u) {
+      const long long n = n0 + (long long)u * V.P;
+      a.x[n] = xn[u] + alpha * pn[u];
+      rn[u] = rn[u] - alpha * qn[u];
+      a.r[n] = rn[u];
+      a.z[n] = dn * rn[u];
+    }
+  }
 #pragma unroll
   for (int u = 0; u < FS; ++u) {
+    if (plain) continue;
     rn[u] = 0.0f;
     const int j = ij.y + r0 + u;
     if (i <= V.nx && j <= V.ny) {
@@ -472,6 +572,44 @@ __global__ void __launch_bounds__(NT) k_mg0_sweep(FineArgs a, const float* zi, f
   const int tid = linear_tid(), col = tid % CTX, r0 = (tid / CTX) * FS;
   const int i = ij.x + col;
   float rv[FS], dv[FS];
+  if (plain_tile(a, V, ij, PROL)) {
+    const int lane = tid & 31;
+    const long long n0 = V.base + (long long)(ij.y + r0) * V.P + i;
+    PlainCols q;
+    plain_load(q, zi, n0, V.P, lane);
+#pragma unroll
+    for (int u = 0; u < FS; ++u) rv[u] = a.r[n0 + (long long)u * V.P];
+    const float d0 = MODE != 1 ? a.dinv0[n0] : 0.0f;
+    if (PROL) {
+      const float* cz = a.c_zb + a.c_off[v];
+      const int w = a.c_dims[v].x + 1;
+      float e[FS + 2];
+      plain_prolong(cz, w, i, ij.y + r0, e);
+#pragma unroll
+      for (int r = 0; r < FS + 2; ++r) q.c[r] += e[r];
+      if (lane == 0 || lane == 31) {
+        plain_prolong(cz, w, lane == 0 ? i - 1 : i + 1, ij.y + r0, e);
+#pragma unroll
+        for (int r = 0; r < FS + 2; ++r) q.e[r] += e[r];
+      }
+    }
+    float y[FS];
+    plain_apply(q, V.kr32, lane, y);
+    float zout[FS];
+#pragma unroll
+    for (int u = 0; u < FS; ++u) {
+      const float rr = rv[u] - y[u];
+      zout[u] = MODE == 1 ? rr : q.c[u + 1] + d0 * rr;
+      zo[n0 + (long long)u * V.P] = zout[u];
+    }
+    if (MODE == 2) {
+      Acc<float> acc;
+      acc.zero();
+      acc.add4(0, rv, zout);
+      block_dot_acc(acc, a.part, sh);
+    }
+    return;
+  }
 #pragma unroll
   for (int u = 0; u < FS; ++u) {
     const int j = ij.y + r0 + u;
@@ -526,6 +664,32 @@ __global__ void __launch_bounds__(NT) k_mg0_apply(FineArgs a) {
   const float* pb = a.sb + 2 * a.B;
   const int tid = linear_tid(), col = tid % CTX, r0 = (tid / CTX) * FS;
   const int i = ij.x + col;
+  if (plain_tile(a, V, ij, false)) {
+    const int lane = tid & 31;
+    const long long n0 = V.base + (long long)(ij.y + r0) * V.P + i;
+    PlainCols q, o;
+    plain_load(q, a.t, n0, V.P, lane);
+    plain_load(o, pold, n0, V.P, lane);
+#pragma unroll
+    for (int r = 0; r < FS + 2; ++r) {
+      q.c[r] = q.c[r] + beta * o.c[r];
+      q.e[r] = q.e[r] + beta * o.e[r];
+    }
+    float y[FS], pp[FS];
+    plain_apply(q, V.kr32, lane, y);
+#pragma unroll
+    for (int u = 0; u < FS; ++u) {
+      const long long n = n0 + (long long)u * V.P;
+      pp[u] = q.c[u + 1];
+      a.q[n] = y[u];
+      pnew[n] = pp[u];
+    }
+    Acc<float> acc;
+    acc.zero();
+    acc.add4(0, pp, y);
+    block_dot_acc(acc, a.part, sh);
+    return;
+  }
   // t + beta p_old is zero at nodes without an unknown; BODY nodes take the body's value
   auto pval = [&](long long n, uint8_t tg) -> float {
     const float f = a.t[n] + beta * pold[n];
@@ -1087,6 +1251,7 @@ void launch_pcg_chunk(Batch& b, int iters, cudaStream_t s) {
   a.m = mesh_view(b);
   a.tile_var = b.tile_cg_var;
   a.tile_ij = b.tile_cg_ij;
+  a.tile_gen = b.tile_cg_gen;
   a.st = b.state;
   a.dinv0 = b.mg_dinv0;
   a.x = b.mg_x;
