@@ -240,18 +240,19 @@ template <> struct Acc<float> {
 #pragma unroll
     for (int u = 0; u < N; ++u) ff_add_prod(v[k], x[u], y[u]);
   }
+  __device__ double warp_sum(int k) {
+    FF s = v[k];
+    s = ff_add(s, FF{0.f, 0.f});   // renormalise
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      FF t{__shfl_xor_sync(0xffffffffu, s.hi, o), __shfl_xor_sync(0xffffffffu, s.lo, o)};
+      s = ff_add(s, t);
+    }
+    return (double)s.hi + (double)s.lo;
+  }
   __device__ void warp_reduce(double out[4]) {
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      FF s = v[k];
-      s = ff_add(s, FF{0.f, 0.f});   // renormalise
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        FF t{__shfl_xor_sync(0xffffffffu, s.hi, o), __shfl_xor_sync(0xffffffffu, s.lo, o)};
-        s = ff_add(s, t);
-      }
-      out[k] = (double)s.hi + (double)s.lo;
-    }
+    for (int k = 0; k < 4; ++k) out[k] = warp_sum(k);
   }
 };
 

@@ -562,21 +562,24 @@ __global__ void k_stiffness(const DevVariant* var, const int* tile_var, const in
                             long long* stats_i, double* detmin, const int* bid, const double2* pcut, int* err) {
   TileCtx c = tile_ctx(var, tile_var, tile_ij);
   const DevVariant& V = var[c.v];
-  __shared__ long long cnt[6];
-  __shared__ double dmin;
+  __shared__ int cnt[6];
+  __shared__ unsigned long long dmin;      // smallest det J, as an integer that orders like the double
   const int tid = linear_tid();
   if (tid < 6) cnt[tid] = 0;
-  if (tid == 0) dmin = 1e300;
+  if (tid == 0) dmin = ~0ull;
   __syncthreads();
+  // (counted and compared per warp first: 256 atomics on one shared word serialise)
+  int what = 0;                            // bit k: counter k
+  double det = 1e300;
   if (c.in) {
     const long long n = c.n;
     const uint8_t t = tag[n];
     const uint8_t kind = t & KIND_MASK;
-    if (kind == K_FREE) atomicAdd((unsigned long long*)&cnt[0], 1ull);
-    if (kind == K_BODY) atomicAdd((unsigned long long*)&cnt[1], 1ull);
-    if (kind == K_INACT) atomicAdd((unsigned long long*)&cnt[2], 1ull);
+    if (kind == K_FREE) what |= 1;
+    if (kind == K_BODY) what |= 2;
+    if (kind == K_INACT) what |= 4;
     if (t & CELL_ACTIVE) {
-      atomicAdd((unsigned long long*)&cnt[3], 1ull);
+      what |= 8;
       const long long idx[4] = {n, n + 1, n + 1 + V.P, n + V.P};
       CutPoly cp;
       cp.n = 0;
@@ -588,14 +591,14 @@ __global__ void k_stiffness(const DevVariant* var, const int* tile_var, const in
       bool disp = false;
       for (int a = 0; a < 4; ++a) disp |= (tag[idx[a]] & DISPLACED) != 0;
       if (cst != CUT_OK) {
-        atomic_min_double(&dmin, -1.0);              // refused cell: the mesh is invalid
+        det = -1.0;                                  // refused cell: the mesh is invalid
       } else if (cp.n == 0 && !disp) {
         // an undisplaced hx-by-hy rectangle: det J = (hx/2)(hy/2) at every Gauss point.
         // The closed-form constants are stored for the resident CG, which reads the
         // coefficients of every cell around a node without looking at tags (inactive cells
         // and those outside the grid hold zeros); every other reader takes the constants
         for (int m = 0; m < 6; ++m) K64[m * Vtot + n] = V.kr64[m];
-        atomic_min_double(&dmin, 0.25 * V.hx * V.hy);
+        det = 0.25 * V.hx * V.hy;
       } else {
         double k6[6], dm;
         if (cp.n > 0) {
@@ -618,15 +621,29 @@ __global__ void k_stiffness(const DevVariant* var, const int* tile_var, const in
         bool differs32 = false;
         for (int m = 0; m < 6; ++m) differs32 |= (float)k6[m] != V.kr32[m];
         tag[n] = t | CELL_GENERAL | (differs32 ? CELL_GEN32 : 0);
-        atomicAdd((unsigned long long*)&cnt[4], 1ull);
-        if (differs32) atomicAdd((unsigned long long*)&cnt[5], 1ull);
-        atomic_min_double(&dmin, dm);
+        what |= 16 | (differs32 ? 32 : 0);
+        det = dm;
       }
     }
   }
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    const int m = __popc(__ballot_sync(0xffffffffu, (what >> k) & 1));
+    if (m && (tid & 31) == 0) atomicAdd(&cnt[k], m);
+  }
+  if (det != det) det = 1e300;             // (a NaN compares below nothing)
+  const long long db = __double_as_longlong(det);
+  unsigned long long key = db < 0 ? ~(unsigned long long)db : (unsigned long long)db | (1ull << 63);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) key = min(key, __shfl_xor_sync(0xffffffffu, key, o));
+  if ((tid & 31) == 0) atomicMin(&dmin, key);
   __syncthreads();
   if (tid < 6 && cnt[tid]) atomicAdd((unsigned long long*)&stats_i[c.v * 6 + tid], (unsigned long long)cnt[tid]);
-  if (tid == 0 && dmin < 1e300) atomic_min_double(&detmin[c.v], dmin);
+  if (tid == 0) {
+    const unsigned long long k = dmin;
+    const double d = k >> 63 ? __longlong_as_double((long long)(k & ~(1ull << 63))) : __longlong_as_double((long long)~k);
+    if (d < 1e300) atomic_min_double(&detmin[c.v], d);
+  }
 }
 
 // 5b. per fused-CG tile: does any cell used by the tile (cells i0-1 .. i0+CTX-1,

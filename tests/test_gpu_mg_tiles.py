@@ -19,7 +19,7 @@ def _case(nx, ny, bc=(D, D, D, D), r=0.4):
 
 
 CASES = {"one_tile": [_case(40, 20, r=0.7)], "no_plain_tile": [_case(130, 40)], "even": [_case(320, 160)],
-         "odd": [_case(321, 161)], "natural": [_case(257, 129, (N, N, D, D))],
+         "odd": [_case(321, 161)], "natural": [_case(256, 129, (N, N, D, D))],
          "natural_odd_tile_edge": [_case(255, 127, (N, N, N, D))], "tile_multiple": [_case(384, 192)],
          "batch": [_case(200, 100), _case(333, 167), _case(96, 48)]}
 
@@ -29,7 +29,7 @@ def test_multigrid_solve_matches_oracle(name):
     from paper_2512_12232_gb300 import api
     cases = CASES[name]
     with api.batch_build(cases) as g:
-        res = api.psi_solve(g, U=1.0, tol=1e-12, precision=api.PF_MIXED, preconditioner="mg")
+        res = api.psi_solve(g, U=1.0, tol=1e-12, precision=api.PF_MIXED, preconditioner="mg", k_max=400)
         psi = res.psi.cpu().numpy()
         for v, c in enumerate(cases):
             assert res.info[v]["status"] == 0 and res.info[v]["rel_true_residual"] <= 1e-12
