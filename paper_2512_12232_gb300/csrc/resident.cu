@@ -35,11 +35,14 @@
 // What bounds it (GB300, 2070 MHz): per iteration about 2 us between a CTA's partial sums and
 // the next alpha (two hops through L2 of 0.4 us, and the first block's FP64 sums and division
 // at 64 cycles a dependent instruction), the rest instruction latency at eight warps per
-// scheduler pair.  Measured, time per CG iteration, streaming kernel -> here: five 403x201
-// channel variants, FP32, 25.5 -> 8.6 us; one 128x64 cylinder, FP64, 14.1 (24 with the idle
-// launches of its chunks) -> 8.4 us; 16 solves of 256x128, FP32, 18.6 -> 11.7 us; one 1024x512
-// grid, FP64, 54 -> 43 us (FP64 arithmetic).  256 variants (62 M nodes): 1.50 -> 1.75 s a
-// solve, hence the limit on the queue.
+// scheduler pair.  In the first block four warps sum the dot products and the other four the
+// bodies' rows, four bodies at a time with eight lanes each: all eight warps taking whole sums
+// in turn made the 12-body variants wait for a second round (five 403x201 channel variants 8.6
+// -> 7.8 us an iteration, one 1024x512 grid in FP64 43 -> 38 us).  Measured, time per CG
+// iteration, streaming kernel -> here: five 403x201 channel variants, FP32, 25.5 -> 7.8 us; one
+// 128x64 cylinder, FP64, 14.1 (24 with the idle launches of its chunks) -> 8.4 us; 16 solves of
+// 256x128, FP32, 18.6 -> 11.2 us; one 1024x512 grid, FP64, 54 -> 38 us (FP64 arithmetic).  256
+// variants (62 M nodes): 1.50 -> 1.75 s a solve, hence the limit on the queue.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -52,6 +55,7 @@ namespace {
 
 constexpr int RNT = 256;                  // threads per CTA
 constexpr int RWARPS = RNT / 32;
+static_assert(RWARPS > 4, "four warps sum the dot products, the others the bodies");
 constexpr int HITER = 3;                  // halo nodes per thread at most
 constexpr int HMAX = HITER * RNT;
 constexpr int NSMAX = 8;                  // strips per block at most
@@ -988,40 +992,49 @@ __global__ void __launch_bounds__(RNT, 2) k_cg_resident(ResArgs<T> g) {
       const int nbu = sh.nbu, parts = sh.parts;
       if (part == 0) {
         // ---- first block: all partial sums, in block order, then the scalars
-        for (int qd = warp; qd < 4 + nbu; qd += RWARPS) {
-          const u64* const all = sh.pw_var + (ep & 1) * g.pw_half + (long long)qd * parts * 2;
-          const int* const list = sh.blist + (long long)(qd - 4) * parts;
-          const int n = qd < 4 ? parts : s_cnt[qd - 4], first = qd < 4 ? 0 : s_first[qd - 4];
+        // (a dot product per warp; of the bodies, which few blocks hold, four per warp)
+        const u64* const now = sh.pw_var + (ep & 1) * g.pw_half;
+        auto wait_sum = [&](const u64* at) {
+          u64 wa, wb;
+          ld_word2(at, wa, wb);
+          int tries = 0;
+          while (!fresh(wa, wb, ep)) {
+            if (give_up(tries)) {
+              gave_up = true;
+              break;
+            }
+            ld_word2(at, wa, wb);
+          }
+          return word_double(wa, wb);
+        };
+        if (warp < 4) {
+          const u64* const all = now + (long long)warp * parts * 2;
           double s = 0.0;
-          for (int pp = lane; pp < n; pp += 128) {
+          for (int pp = lane; pp < parts; pp += 128) {
             u64 wa[4], wb[4];
-            const u64* at[4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              const int e = pp + 32 * u;
-              if (e < n) {
-                at[u] = all + 2 * (qd < 4 ? e : first >= 0 ? s_list[first + e] : list[e]);
-                ld_word2(at[u], wa[u], wb[u]);
-              }
-            }
+            for (int u = 0; u < 4; ++u)
+              if (pp + 32 * u < parts) ld_word2(all + 2 * (pp + 32 * u), wa[u], wb[u]);
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              if (pp + 32 * u < n) {
-                int tries = 0;
-                while (!fresh(wa[u], wb[u], ep)) {
-                  if (give_up(tries)) {
-                    gave_up = true;
-                    break;
-                  }
-                  ld_word2(at[u], wa[u], wb[u]);
-                }
-                s += word_double(wa[u], wb[u]);
-              }
-            }
+            for (int u = 0; u < 4; ++u)
+              if (pp + 32 * u < parts)
+                s += fresh(wa[u], wb[u], ep) ? word_double(wa[u], wb[u]) : wait_sum(all + 2 * (pp + 32 * u));
           }
 #pragma unroll
           for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-          if (lane == 0) s_tot[qd] = s;
+          if (lane == 0) s_tot[warp] = s;
+        } else {
+          for (int k0 = 4 * (warp - 4); k0 < nbu; k0 += 4 * (RWARPS - 4)) {
+            const int k = k0 + (lane >> 3), n = k < nbu ? s_cnt[k] : 0, first = k < nbu ? s_first[k] : 0;
+            const u64* const all = now + (long long)(4 + k) * parts * 2;
+            double s = 0.0;
+            for (int e = lane & 7; e < n; e += 8)
+              s += wait_sum(all + 2 * (first >= 0 ? s_list[first + e] : sh.blist[(long long)k * parts + e]));
+            __syncwarp();
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if ((lane & 7) == 0 && k < nbu) s_tot[4 + k] = s;
+          }
         }
         if (gave_up) {
           atomicExch(g.err, 1);

@@ -85,3 +85,20 @@ def test_resident_iteration_cap(api):
         res = api.psi_solve(g, U=1.0, tol=1e-12, precision=api.PF_MIXED, k_max=11, raise_on_failure=False)
         assert res.info[0]["iters"] == 11 and res.info[0]["status"] == 3   # PF_ENOT_CONVERGED
         assert np.all(np.isfinite(res.psi.cpu().numpy()))
+
+
+@pytest.mark.parametrize("rows,cols", [(4, 4), (5, 7)])
+def test_resident_solve_with_many_bodies(api, rows, cols):
+    """The first block sums sixteen bodies' rows at a time: as many, and three rounds of them,
+    with bodies in one block and across several."""
+    bodies = [[-3.4 + 6.8 * i / (cols - 1) + 0.011, -1.5 + 3.0 * j / (rows - 1) + 0.007, 0.23]
+              for j in range(rows) for i in range(cols)]
+    c = _case(201, 101, bodies)
+    m = OM.build_mesh(c.grid, c.bodies, c.sweeps, c.bc)
+    s = OSY.assemble(m, 1.0)
+    u, psi = OS.solve_direct(s)
+    with api.mesh_build(c.grid, c.bodies, c.sweeps, c.bc) as g:
+        for p, tol, bound in ((api.PF_FP64, 1e-13, 1e-10), (api.PF_MIXED, 1e-12, 1e-6)):
+            res = api.psi_solve(g, U=1.0, tol=tol, precision=p)
+            assert rel_l2(res.psi.cpu().numpy(), psi) <= bound
+            np.testing.assert_allclose(res.body_psi, u[s.n_free:], rtol=0, atol=10 * bound)
