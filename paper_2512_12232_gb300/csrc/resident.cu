@@ -36,12 +36,12 @@
 // the next alpha (two hops through L2 of 0.4 us, and the first block's FP64 sums and division
 // at 64 cycles a dependent instruction), the rest instruction latency at eight warps per
 // scheduler pair.  In the first block four warps sum the dot products and the other four the
-// bodies' rows, four bodies at a time with eight lanes each: all eight warps taking whole sums
-// in turn made the 12-body variants wait for a second round (five 403x201 channel variants 8.6
+// bodies' rows, four bodies at a time with eight lanes each: with all eight warps taking whole sums
+// in turn, variants of five and more bodies waited for a second round (five 403x201 channels 8.6
 // -> 7.8 us an iteration, one 1024x512 grid in FP64 43 -> 38 us).  Measured, time per CG
 // iteration, streaming kernel -> here: five 403x201 channel variants, FP32, 25.5 -> 7.8 us; one
 // 128x64 cylinder, FP64, 14.1 (24 with the idle launches of its chunks) -> 8.4 us; 16 solves of
-// 256x128, FP32, 18.6 -> 11.2 us; one 1024x512 grid, FP64, 54 -> 38 us (FP64 arithmetic).  256
+// 256x128, FP32, 18.6 -> 8.7 us; one 1024x512 grid, FP64, 54 -> 38 us (FP64 arithmetic).  256
 // variants (62 M nodes): 1.50 -> 1.75 s a solve, hence the limit on the queue.
 #include <algorithm>
 #include <cmath>
@@ -1225,42 +1225,73 @@ struct Cutter {
   int tx = 0, ty = 0;                  // 64 x 16 tiles
   std::vector<uint8_t> stored;         // [ty][tx] some operator row needs stored coefficients
 
-  // one column part: appends (j0, ha, gen); false if the exchange lists would overflow
-  bool column(int i0, int w, int ns, int rows, int grows, std::vector<RItem>* out, int& parts, double& slots) const {
-    const int unit = ns * H, last = std::min(W - 1, i0 + w - 1);
-    int j = 0;
+  // rows to which tile rows of column part [i0, i0 + w) without stored coefficients run on: 0
+  // where the tile row has stored ones
+  void runs(int i0, int w, std::vector<int>& plain_to) const {
+    const int last = std::min(W - 1, i0 + w - 1);
+    plain_to.assign(ty, 0);
+    for (int t = ty - 1; t >= 0; --t) {
+      bool st = false;
+      for (int c = i0 / CTX; c <= last / CTX && !st; ++c) st = stored[(size_t)t * tx + c] != 0;
+      if (!st) plain_to[t] = t + 1 < ty && plain_to[t + 1] ? plain_to[t + 1] : std::min(R, (t + 1) * CTY);
+    }
+  }
+  struct Part { int i0, w, ns, unit, rows, grows; };
+
+  // Blocks of a column part from row j down, each as high as it may be: their number, and their
+  // rows in `slots`.  Where a plain run ends in a low block, that may join the stored block below,
+  // and the last block of a stored run may stop with it or run on.  Of these two ways the one
+  // with fewer blocks is taken, `forks` times per column part (once: 16 grids of 257x129 nodes
+  // with an airfoil each need 256 blocks in place of 320, so that all of them fit the chip; more
+  // often costs host time that doubles with every fork and gains under 2 % of the blocks).
+  int down(const Part& c, const std::vector<int>& plain_to, int j, int forks, double& slots, std::vector<RItem>* out) const {
+    int n = 0;
     while (j < R) {
-      int t = j / CTY;
-      auto row_stored = [&](int t1) {
-        for (int c = i0 / CTX; c <= last / CTX; ++c)
-          if (stored[(size_t)t1 * tx + c]) return true;
-        return false;
+      const int end = plain_to[j / CTY], left = (R - j + c.unit - 1) / c.unit;
+      const int full = std::max(2, std::min(c.grows, left));
+      int ha = 0, gen = 1;
+      auto fewer = [&](int h1, int h2) {         // blocks below a block of h1 rows against one of h2
+        double s = 0.0;
+        return down(c, plain_to, j + c.unit * h1, forks, s, nullptr) < down(c, plain_to, j + c.unit * h2, forks, s, nullptr);
       };
-      int end, ha, gen;
-      if (row_stored(t)) {
-        while (t < ty && row_stored(t)) ++t;
-        end = std::min(R, t * CTY);
-        const int need = end - j, m = (need + unit * grows - 1) / (unit * grows);
-        ha = std::max(2, (need + unit * m - 1) / (unit * m));
-        gen = 1;
-      } else {
-        while (t < ty && !row_stored(t)) ++t;
-        end = std::min(R, t * CTY);
-        const int run = end - j, m = (run + unit * rows - 1) / (unit * rows);
-        ha = std::max(2, (run + unit * m - 1) / (unit * m));
-        gen = 0;
-        if (end < R && unit * ha * m > run) ha = run / (unit * m);   // stay clear of the stored ones
-        if (ha < 2) {
-          ha = 2;
-          gen = 1;
+      if (end) {
+        const int fit = end == R ? left : (end - j) / c.unit;
+        ha = std::min(fit, c.rows);
+        if (fit > ha && fit - ha < 2 && ha > 3) ha = fit - 2;       // leave no single row
+        if (end == R) ha = std::max(ha, 2);
+        if (ha >= 2) gen = 0;
+        if (!gen && end < R && fit <= c.rows && forks > 0) {
+          --forks;
+          gen = fewer(full, ha);
         }
       }
-      if (2 * (w + 2) + 2 * unit * ha > HMAX || ha > (gen ? grows : rows)) return false;
-      if (out) out->push_back(RItem{0, 0, i0, w, j, ns, ha, gen});
-      ++parts;
+      if (gen) {
+        ha = full;
+        int t = j / CTY;
+        while (t < ty && plain_to[t]) ++t;                  // (the plain rest that joined)
+        while (t < ty && !plain_to[t]) ++t;
+        const int need = std::max(2, (std::min(R, t * CTY) - j + c.unit - 1) / c.unit);
+        if (need < full && forks > 0) {
+          --forks;
+          if (!fewer(full, need)) ha = need;
+        }
+      }
+      if (out) out->push_back(RItem{0, 0, c.i0, c.w, j, c.ns, ha, gen});
+      ++n;
       slots += ha;
-      j += unit * ha;
+      j += c.unit * ha;
     }
+    return n;
+  }
+
+  // one column part: appends (j0, ha, gen); false if the exchange lists would overflow
+  bool column(int i0, int w, int ns, int rows, int grows, std::vector<RItem>* out, int& parts, double& slots) const {
+    const int unit = ns * H, fit = (HMAX - 2 * (w + 2)) / (2 * unit);
+    if (fit < 2) return false;
+    const Part c{i0, w, ns, unit, std::min(rows, fit), std::min(grows, fit)};
+    std::vector<int> plain_to;
+    runs(i0, w, plain_to);
+    parts += down(c, plain_to, 0, 1, slots, out);
     return true;
   }
 
@@ -1295,6 +1326,13 @@ struct Cutter {
     return true;
   }
 };
+
+void free_plan(Batch& b, ResPlan& R) {
+  for (void* p : {R.d_var, R.d_items, (void*)R.d_ctrl, (void*)R.d_epoch, (void*)R.d_pw, (void*)R.d_bc,
+                  (void*)R.d_pbm, (void*)R.d_blist})
+    if (p) dev_free(b, p);
+  R = ResPlan{};
+}
 
 }  // namespace
 
@@ -1355,13 +1393,13 @@ bool resident_ready(Batch& b, int precision) {
     if (fl[t] & bit) cut[var[t]].stored[(size_t)(ij[t].y / CTY) * cut[var[t]].tx + ij[t].x / CTX] = 1;
   std::vector<std::vector<RItem>> blocks(b.nv);
   long long total = 0;
-  auto plan = [&](int cap, int gcap, int threads) {
+  auto plan = [&](int cap, int gcap, int threads, long long most) {
     total = 0;
-    for (int v = 0; v < b.nv; ++v) {
+    for (int v = 0; v < b.nv && total <= most; ++v) {
       if (!cut[v].best(cap, std::max(2, std::min(grows, gcap)), threads, blocks[v])) return false;
       total += (long long)blocks[v].size();
     }
-    return true;
+    return total <= most;
   };
   // all at once: the cut whose iteration is estimated shortest.  An iteration's fixed part costs
   // about as much as five rows; a row with stored coefficients 1.6 times (FP64: 1.5 times) a row
@@ -1373,7 +1411,7 @@ bool resident_ready(Batch& b, int precision) {
       for (int gc = std::max(2, cap / 2); gc <= std::min(cap, grows); ++gc) {
         if (nodes > (double)G * threads * H * cap) continue;
         const double cost = (5.0 + std::max((double)cap, (f64 ? 1.5 : 1.6) * gc)) * threads / RNT;
-        if (cost >= best_cost || !plan(cap, gc, threads) || total > G) continue;
+        if (cost >= best_cost || !plan(cap, gc, threads, G)) continue;
         const double c2 = cost * (double)((total + b.nsm - 1) / b.nsm);
         if (c2 < best_cost) {
           best_cost = c2;
@@ -1383,9 +1421,9 @@ bool resident_ready(Batch& b, int precision) {
         }
       }
   const bool spread = best_cap > 0;
-  if (spread) plan(best_cap, best_gcap, best_threads);
+  if (spread) plan(best_cap, best_gcap, best_threads, G);
   // else the largest blocks, and the variants queue
-  if (!spread && (nodes > 2.0 * G * RNT * H * rows || !plan(rows, grows, RNT) || total > 2 * G)) return false;
+  if (!spread && (nodes > 2.0 * G * RNT * H * rows || !plan(rows, grows, RNT, 2 * G))) return false;
   size_t most = 0;
   for (auto& x : blocks) most = std::max(most, x.size());
   if ((long long)most > G || total > (1 << 24)) return false;
@@ -1416,14 +1454,21 @@ bool resident_ready(Batch& b, int precision) {
   R.pw_half = total * R.qs * 2;
   const size_t WPV = f64 ? 2 : 1;
   const size_t bc_words = (size_t)b.nv * 2 * (R.qs - 1) * WPV;
-  R.d_var = dev_alloc(b, b.nv * sizeof(RVar));
-  R.d_items = dev_alloc(b, items.size() * sizeof(RItem));
-  R.d_ctrl = (int*)dev_alloc(b, (1 + b.nv) * sizeof(int));
-  R.d_epoch = (unsigned*)dev_alloc(b, b.nv * sizeof(unsigned));
-  R.d_pw = (unsigned long long*)dev_alloc(b, 2 * R.pw_half * sizeof(u64));
-  R.d_bc = (unsigned long long*)dev_alloc(b, bc_words * sizeof(u64));
-  R.d_pbm = (unsigned long long*)dev_alloc(b, total * sizeof(u64));
-  R.d_blist = (int*)dev_alloc(b, std::max<long long>(1, total * nbm) * sizeof(int));
+  try {
+    R.d_var = dev_alloc(b, b.nv * sizeof(RVar));
+    R.d_items = dev_alloc(b, items.size() * sizeof(RItem));
+    R.d_ctrl = (int*)dev_alloc(b, (1 + b.nv) * sizeof(int));
+    R.d_epoch = (unsigned*)dev_alloc(b, b.nv * sizeof(unsigned));
+    R.d_pw = (unsigned long long*)dev_alloc(b, 2 * R.pw_half * sizeof(u64));
+    R.d_bc = (unsigned long long*)dev_alloc(b, bc_words * sizeof(u64));
+    R.d_pbm = (unsigned long long*)dev_alloc(b, total * sizeof(u64));
+    R.d_blist = (int*)dev_alloc(b, std::max<long long>(1, total * nbm) * sizeof(int));
+  } catch (const Error& e) {
+    if (e.code != PF_ENOMEM) throw;
+    free_plan(b, R);                     // no room for the exchange buffers: the streaming kernel solves
+    R.made = true;
+    return false;
+  }
   PF_CUDA(cudaMemcpyAsync(R.d_var, vars.data(), b.nv * sizeof(RVar), cudaMemcpyHostToDevice, b.stream));
   PF_CUDA(cudaMemcpyAsync(R.d_items, items.data(), items.size() * sizeof(RItem), cudaMemcpyHostToDevice, b.stream));
   PF_CUDA(cudaMemsetAsync(R.d_epoch, 0, b.nv * sizeof(unsigned), b.stream));
@@ -1436,12 +1481,7 @@ bool resident_ready(Batch& b, int precision) {
 
 // The plan is made again on the next solve (node coordinates were replaced).
 void drop_resident(Batch& b) {
-  for (ResPlan& R : b.res) {
-    for (void* p : {R.d_var, R.d_items, (void*)R.d_ctrl, (void*)R.d_epoch, (void*)R.d_pw, (void*)R.d_bc,
-                    (void*)R.d_pbm, (void*)R.d_blist})
-      if (p) dev_free(b, p);
-    R = ResPlan{};
-  }
+  for (ResPlan& R : b.res) free_plan(b, R);
 }
 
 template <typename T>

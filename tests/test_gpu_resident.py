@@ -102,3 +102,63 @@ def test_resident_solve_with_many_bodies(api, rows, cols):
             res = api.psi_solve(g, U=1.0, tol=tol, precision=p)
             assert rel_l2(res.psi.cpu().numpy(), psi) <= bound
             np.testing.assert_allclose(res.body_psi, u[s.n_free:], rtol=0, atol=10 * bound)
+
+
+def test_resident_blocks_join_short_plain_runs(api):
+    """Sixteen variants whose rows of undisplaced cells above and below the body are too few for
+    blocks of their own: they join the neighbouring blocks, and the batch fits at once."""
+    cases = [_case(256, 128, [[0.13 + 0.004 * k, 0.07 - 0.01 * k, 0.25]], 40) for k in range(16)]
+    with api.batch_build(cases) as g:
+        for p, tol, bound in ((api.PF_FP64, 1e-13, 1e-10), (api.PF_MIXED, 1e-12, 1e-6)):
+            res = api.psi_solve(g, U=1.0, tol=tol, precision=p)
+            psi = res.psi.cpu().numpy()
+            for v in (0, 7, 15):
+                c = cases[v]
+                m = OM.build_mesh(c.grid, c.bodies, c.sweeps, c.bc)
+                _, ref = OS.solve_direct(OSY.assemble(m, 1.0))
+                assert rel_l2(psi[g.node_offsets[v]:g.node_offsets[v + 1]], ref) <= bound, v
+
+
+def test_solve_without_room_for_the_exchange_buffers(api):
+    """Each allocation of a handle's first solve is refused in turn.  Where it was one of the eight
+    of the exchange between blocks, the streaming kernel solves; the others end in PF_ENOMEM."""
+    import torch
+    from paper_2512_12232_gb300 import _lib
+    lib = _lib.load()
+    made, refused = [0], [-1]
+
+    @_lib.ALLOC_FN
+    def alloc(nbytes, stream, ctx):
+        made[0] += 1
+        if made[0] - 1 == refused[0]:
+            return None
+        return torch.cuda.caching_allocator_alloc(int(nbytes), torch.cuda.current_device(), int(stream or 0))
+
+    @_lib.FREE_FN
+    def free(ptr, stream, ctx):
+        torch.cuda.caching_allocator_delete(int(ptr))
+
+    c = CASES["ragged"][0]
+    ref, _ = _reference("ragged", 0)
+    streamed = 0
+    assert lib.pf_set_allocator(alloc, free, None) == _lib.PF_OK
+    try:
+        with api.mesh_build(c.grid, c.bodies, c.sweeps, c.bc) as g:
+            built = made[0]
+            res = api.psi_solve(g, U=1.0, tol=1e-13, precision=api.PF_FP64)
+            total = made[0]
+            assert g.timing()["cg_launches"] == res.info[0]["iters"]
+        for k in range(built, total):
+            made[0], refused[0] = 0, k
+            with api.mesh_build(c.grid, c.bodies, c.sweeps, c.bc) as g:
+                try:
+                    res = api.psi_solve(g, U=1.0, tol=1e-13, precision=api.PF_FP64)
+                except _lib.PfError as e:
+                    assert "PF_ENOMEM" in str(e)
+                    continue
+                assert rel_l2(res.psi.cpu().numpy(), ref) <= 1e-10
+                # (the streaming kernel runs whole chunks of launches, more than there are iterations)
+                streamed += g.timing()["cg_launches"] > res.info[0]["iters"]
+    finally:
+        lib.pf_set_allocator(_lib.ALLOC_FN(), _lib.FREE_FN(), None)
+    assert streamed == 8
