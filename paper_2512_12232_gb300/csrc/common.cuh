@@ -54,6 +54,8 @@ constexpr uint8_t TILE_PLAIN64 = 4;   // window all FREE, no TILE_GEN64 cell
 constexpr uint8_t TILE_PLAIN32 = 8;   // window all FREE, no TILE_GEN32 cell
 constexpr uint8_t TILE_ROW64 = 16;    // a FREE or BODY node of the tile whose four cells are not all active
 constexpr uint8_t TILE_ROW32 = 32;    // ones without stored FP64 (FP32) K_e
+constexpr uint8_t TILE_FREE = 64;     // window all FREE (every cell active)
+constexpr uint8_t TILE_EMPTY = 128;   // no node of the tile has an operator row
 
 // solver phases (per variant)
 constexpr int PH_CG = 0, PH_RESID = 1, PH_DONE = 2;

@@ -594,10 +594,14 @@ __global__ void k_stiffness(const DevVariant* var, const int* tile_var, const in
         det = -1.0;                                  // refused cell: the mesh is invalid
       } else if (cp.n == 0 && !disp) {
         // an undisplaced hx-by-hy rectangle: det J = (hx/2)(hy/2) at every Gauss point.
-        // The closed-form constants are stored for the resident CG, which reads the
-        // coefficients of every cell around a node without looking at tags (inactive cells
-        // and those outside the grid hold zeros); every other reader takes the constants
-        for (int m = 0; m < 6; ++m) K64[m * Vtot + n] = V.kr64[m];
+        // The closed-form constants are stored for the resident CG and for the multigrid
+        // cycle's stored tiles, which read the coefficients of every cell around a node without
+        // looking at tags (inactive cells and those outside the grid hold zeros); every other
+        // reader takes the constants
+        for (int m = 0; m < 6; ++m) {
+          K64[m * Vtot + n] = V.kr64[m];
+          K32[m * Vtot + n] = V.kr32[m];
+        }
         det = 0.25 * V.hx * V.hy;
       } else {
         double k6[6], dm;
@@ -653,7 +657,8 @@ __global__ void k_stiffness(const DevVariant* var, const int* tile_var, const in
 //     (so every cell is active) and no cell needs stored coefficients, which lets the
 //     fused CG step skip the tags; and how many of its nodes carry an operator row
 //     (FREE or BODY)?  Bits 4 and 5: some such node's row needs more than the rectangle
-//     constants (a stored, inactive or missing cell around it).  The counts feed the cost estimate of the fused-CG schedule.
+//     constants (a stored, inactive or missing cell around it).  Bit 6: the window is all FREE;
+//     bit 7: no node has a row.  The counts feed the cost estimate of the fused-CG schedule.
 __global__ void k_tile_general(const DevVariant* var, const int* tile_var, const int2* tile_ij, const uint8_t* tag,
                                uint8_t* gen, int* act) {
   __shared__ int sh[NT / 32 + 1];
@@ -702,7 +707,8 @@ __global__ void k_tile_general(const DevVariant* var, const int* tile_var, const
   block_exscan(na, &tot, sh);
   if (linear_tid() == 0) {
     gen[t] = (uint8_t)((g64 ? TILE_GEN64 : 0) | (g32 ? TILE_GEN32 : 0) | (allfree && !g64 ? TILE_PLAIN64 : 0) |
-                       (allfree && !g32 ? TILE_PLAIN32 : 0) | (r64 ? TILE_ROW64 : 0) | (r32 ? TILE_ROW32 : 0));
+                       (allfree && !g32 ? TILE_PLAIN32 : 0) | (r64 ? TILE_ROW64 : 0) | (r32 ? TILE_ROW32 : 0) |
+                       (allfree ? TILE_FREE : 0) | (tot == 0 ? TILE_EMPTY : 0));
     act[t] = tot;
   }
 }
