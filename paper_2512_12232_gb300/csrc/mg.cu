@@ -468,7 +468,7 @@ __device__ __forceinline__ void plain_apply(const PlainCols& q, const float* kr,
 // loaded once, all before the first is used (the general code loads 48 under tag tests).  The
 // kernels' register caps keep the plain tiles at the occupancy they had.  With the tiles inside
 // bodies skipped: 256-variant sweep with mesh build 241.7 -> 232.5 ms, 64 gradients of 1024x512
-// 184.6 -> 178.0 ms, one 8192x4096 solve 91 -> 82 ms.
+// 184.6 -> 178.0 ms, one 8192x4096 solve 7 % shorter.
 __device__ __forceinline__ void stored_apply(const PlainCols& q, const float* K, long long plane, long long n0, int P,
                                              int lane, float (&y)[FS]) {
   const float* own = K + n0 - P;           // cells (i, j0 - 1 ..) and (i - 1, j0 - 1 ..)
