@@ -38,10 +38,10 @@
 // scheduler pair.  In the first block four warps sum the dot products and the other four the
 // bodies' rows, four bodies at a time with eight lanes each: with all eight warps taking whole sums
 // in turn, variants of five and more bodies waited for a second round (five 403x201 channels 8.6
-// -> 7.8 us an iteration, one 1024x512 grid in FP64 43 -> 38 us).  Measured, time per CG
-// iteration, streaming kernel -> here: five 403x201 channel variants, FP32, 25.5 -> 7.8 us; one
-// 128x64 cylinder, FP64, 14.1 (24 with the idle launches of its chunks) -> 8.4 us; 16 solves of
-// 256x128, FP32, 18.6 -> 8.7 us; one 1024x512 grid, FP64, 54 -> 38 us (FP64 arithmetic).  256
+// -> 7.7 us an iteration, one 1024x512 grid in FP64 43 -> 40 us).  Measured, time per CG
+// iteration, streaming kernel -> here: five 403x201 channel variants, FP32, 25.5 -> 7.7 us; one
+// 128x64 cylinder, FP64, 14.1 (24 with the idle launches of its chunks) -> 8.0 us; 16 solves of
+// 256x128, FP32, 18.6 -> 8.7 us; one 1024x512 grid, FP64, 54 -> 40 us (FP64 arithmetic).  256
 // variants (62 M nodes): 1.50 -> 1.75 s a solve, hence the limit on the queue.
 #include <algorithm>
 #include <cmath>
