@@ -46,9 +46,12 @@ struct CgConfig {                  // persistent grid + schedule of one fused-CG
 // How a batch runs with its CG state on the chip (resident.cu), per precision.
 struct ResPlan {
   bool made = false, ok = false;     // the plan was looked for; the batch fits
+  bool open = false;                 // a solve has launched and not come to its end: d_pw and d_bc may hold
+                                     // words numbered past d_epoch
   size_t smem = 0;                   // dynamic shared memory of a CTA
   int grid = 0, n_items = 0, qs = 0; // CTAs, (variant, block) items, sums per block
   long long pw_half = 0;             // words of one parity of d_pw
+  size_t bc_words = 0;               // words of d_bc
   void *d_var = nullptr, *d_items = nullptr;
   int* d_ctrl = nullptr;             // [1 + nv] ticket, started CTAs per variant
   unsigned* d_epoch = nullptr;       // [nv] number of the last exchange
@@ -277,6 +280,7 @@ void body_values(Batch& b, std::vector<double>& C);
 // resident.cu
 bool resident_ready(Batch& b, int precision);
 void launch_resident(Batch& b, int precision, int max_it);
+void end_resident(Batch& b, int precision);
 void drop_resident(Batch& b);
 
 // mg.cu

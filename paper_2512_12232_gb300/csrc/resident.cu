@@ -383,9 +383,11 @@ __global__ void __launch_bounds__(RNT, 2) k_cg_resident(ResArgs<T> g) {
     int P, w, bh, i0, j0, nx, ny, nbu, parts, see;
   } sh;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid == 0) s_abort = 0;
+  // (a wait that gave up in the launch before: its words are not to be continued)
+  if (tid == 0) s_abort = *(volatile int*)g.err != 0;
   for (;;) {
     __syncthreads();
+    if (s_abort) return;
     if (tid == 0) s_item = atomicAdd(g.ticket, 1);
     __syncthreads();
     const int item = s_item;
@@ -1334,6 +1336,15 @@ void free_plan(Batch& b, ResPlan& R) {
   R = ResPlan{};
 }
 
+// Exchange numbers start again at 1: no word carries one.  (The q words lie in the state
+// records, which every solve clears.)
+void clear_exchange(Batch& b, ResPlan& R) {
+  PF_CUDA(cudaMemsetAsync(R.d_epoch, 0, b.nv * sizeof(unsigned), b.stream));
+  PF_CUDA(cudaMemsetAsync(R.d_pw, 0, 2 * R.pw_half * sizeof(u64), b.stream));
+  PF_CUDA(cudaMemsetAsync(R.d_bc, 0, R.bc_words * sizeof(u64), b.stream));
+  R.open = false;
+}
+
 }  // namespace
 
 // Can this batch's CG run with its state on the chip, and how is it cut?  Made once per
@@ -1344,7 +1355,11 @@ void free_plan(Batch& b, ResPlan& R) {
 // take the streaming kernel of solver.cu: it is then bound by bytes, no longer by latency.
 bool resident_ready(Batch& b, int precision) {
   ResPlan& R = b.res[precision];
-  if (R.made) return R.ok;
+  if (R.made) {
+    // after a solve that was broken off (a wait that gave up) the last numbers in use are not known
+    if (R.ok && R.open) clear_exchange(b, R);
+    return R.ok;
+  }
   R.made = true;
   R.ok = false;
   const bool f64 = precision == PF_FP64;
@@ -1453,14 +1468,14 @@ bool resident_ready(Batch& b, int precision) {
   R.qs = 4 + nbm;
   R.pw_half = total * R.qs * 2;
   const size_t WPV = f64 ? 2 : 1;
-  const size_t bc_words = (size_t)b.nv * 2 * (R.qs - 1) * WPV;
+  R.bc_words = (size_t)b.nv * 2 * (R.qs - 1) * WPV;
   try {
     R.d_var = dev_alloc(b, b.nv * sizeof(RVar));
     R.d_items = dev_alloc(b, items.size() * sizeof(RItem));
     R.d_ctrl = (int*)dev_alloc(b, (1 + b.nv) * sizeof(int));
     R.d_epoch = (unsigned*)dev_alloc(b, b.nv * sizeof(unsigned));
     R.d_pw = (unsigned long long*)dev_alloc(b, 2 * R.pw_half * sizeof(u64));
-    R.d_bc = (unsigned long long*)dev_alloc(b, bc_words * sizeof(u64));
+    R.d_bc = (unsigned long long*)dev_alloc(b, R.bc_words * sizeof(u64));
     R.d_pbm = (unsigned long long*)dev_alloc(b, total * sizeof(u64));
     R.d_blist = (int*)dev_alloc(b, std::max<long long>(1, total * nbm) * sizeof(int));
   } catch (const Error& e) {
@@ -1471,9 +1486,7 @@ bool resident_ready(Batch& b, int precision) {
   }
   PF_CUDA(cudaMemcpyAsync(R.d_var, vars.data(), b.nv * sizeof(RVar), cudaMemcpyHostToDevice, b.stream));
   PF_CUDA(cudaMemcpyAsync(R.d_items, items.data(), items.size() * sizeof(RItem), cudaMemcpyHostToDevice, b.stream));
-  PF_CUDA(cudaMemsetAsync(R.d_epoch, 0, b.nv * sizeof(unsigned), b.stream));
-  PF_CUDA(cudaMemsetAsync(R.d_pw, 0, 2 * R.pw_half * sizeof(u64), b.stream));
-  PF_CUDA(cudaMemsetAsync(R.d_bc, 0, bc_words * sizeof(u64), b.stream));
+  clear_exchange(b, R);
   PF_CUDA(cudaStreamSynchronize(b.stream));
   R.ok = true;
   return true;
@@ -1518,6 +1531,7 @@ static void launch(Batch& b, ResPlan& R, State4<T>* const st[2], T* sb, int max_
   a.poll_limit = b.test_drop ? 1024 : MBAR_POLL_LIMIT;
   a.test_drop = b.test_drop;
   a.max_it = max_it;
+  R.open = true;
   PF_CUDA(cudaMemsetAsync(R.d_ctrl, 0, (1 + b.nv) * sizeof(int), b.stream));
   PF_CUDA(cudaFuncSetAttribute(kernel<T>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)R.smem));
   void* args[] = {&a};
@@ -1525,11 +1539,14 @@ static void launch(Batch& b, ResPlan& R, State4<T>* const st[2], T* sb, int max_
 }
 
 // Every variant in the CG phase runs its CG to the inner stopping test, or for max_it
-// iterations (one launch).
+// iterations (one launch).  The caller ends the solve with end_resident once every launch
+// has come to its end without a wait that gave up.
 void launch_resident(Batch& b, int precision, int max_it) {
   ResPlan& R = b.res[precision];
   if (precision == PF_FP64) launch<double>(b, R, b.st64, b.sb64, max_it);
   else launch<float>(b, R, b.st32, b.sb32, max_it);
 }
+
+void end_resident(Batch& b, int precision) { b.res[precision].open = false; }
 
 }  // namespace pfq4

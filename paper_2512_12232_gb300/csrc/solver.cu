@@ -2191,7 +2191,9 @@ pf_status solve_core(Batch& b, double U, const pf_solve_opts& o, double* dev_psi
     res_ms += ms2;
     if (!resident) launches += chunk;
     rlaunches += 1;
-    if (hdone[2 * k + 1]) throw Error{PF_ETIMEOUT, "a bounded wait in the CG kernel gave up (TMA tile not delivered)"};
+    if (hdone[2 * k + 1])
+      throw Error{PF_ETIMEOUT, resident ? "a bounded wait in the resident CG kernel gave up (a block's exchanged values did not arrive)"
+                                        : "a bounded wait in the CG kernel gave up (TMA tile not delivered)"};
     if (hdone[2 * k] >= b.nv) {
       finished = true;
       return;
@@ -2231,6 +2233,7 @@ pf_status solve_core(Batch& b, double U, const pf_solve_opts& o, double* dev_psi
   std::vector<VarState> fin(b.nv);
   PF_CUDA(cudaMemcpyAsync(fin.data(), b.state, b.nv * sizeof(VarState), cudaMemcpyDeviceToHost, s));
   PF_CUDA(cudaStreamSynchronize(s));
+  if (resident) end_resident(b, prec);
   float tot = 0;
   PF_CUDA(cudaEventElapsedTime(&tot, b.ev[3], b.ev[4]));
   b.solved = true;
