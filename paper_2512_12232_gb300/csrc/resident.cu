@@ -39,9 +39,9 @@
 // bodies' rows, four bodies at a time with eight lanes each: with all eight warps taking whole sums
 // in turn, variants of five and more bodies waited for a second round (five 403x201 channels 8.6
 // -> 7.7 us an iteration, one 1024x512 grid in FP64 43 -> 40 us).  Measured, time per CG
-// iteration, streaming kernel -> here: five 403x201 channel variants, FP32, 25.5 -> 7.7 us; one
+// iteration, streaming kernel -> here: five 403x201 channel variants, FP32, 25.5 -> 8.1 us; one
 // 128x64 cylinder, FP64, 14.1 (24 with the idle launches of its chunks) -> 8.0 us; 16 solves of
-// 256x128, FP32, 18.6 -> 8.7 us; one 1024x512 grid, FP64, 54 -> 40 us (FP64 arithmetic).  256
+// 256x128, FP32, 18.6 -> 8.9 us; one 1024x512 grid, FP64, 54 -> 40 us (FP64 arithmetic).  256
 // variants (62 M nodes): 1.50 -> 1.75 s a solve, hence the limit on the queue.
 #include <algorithm>
 #include <cmath>
@@ -121,86 +121,81 @@ template <> struct VT<double> {
 };
 
 // ---------------------------------------------------------------- dot products of one iteration
-// FP32: each product is added exactly.  An accumulator s starts at 1.5 M, M a power of two so
-// large that s stays in [M, 2 M): every s is then a multiple of u = 2^-23 M, t = fma(x, y, s) is
-// s plus x y rounded to that grid, t - s is that rounded product exactly, and fma(x, y, -(t - s))
-// the rest, which goes to a second accumulator l: four packed operations per product, against
-// ten for TwoProd + TwoSum.  M is the same in all lanes of a warp (from its largest |r|, |p| and
-// |q|), so the accumulators of the warp add up as integers: the bits of s count units of u, l is
-// taken in units of 2^-20 u, and one integer reduction instruction per word sums the warp
-// without rounding.  What is lost is below 2^-37 of the largest product of a warp of up to
-// 1024: as for a two-float accumulation, about 2^-45 of the sum.  Only values that are not
-// finite make an accumulator leave [M, 2 M); the sum is then NaN.
+// FP32: the two-float accumulation of k_cg (ff_add_prod), on both halves of a strip at a time.
+// Every product is split exactly (TwoProd), added with TwoSum, and the two errors go to the low
+// word: ten packed operations per product, about 2^-48 relative error per addition.  (Sums on a
+// grid fixed per warp took four, and 0.4 us less an iteration of five 403x201 channels, but kept
+// 6e-12 of sum |p q| where magnitudes are spread and lost |r| below 1e-19 a decade earlier.)
 template <typename T> struct Dots;
 template <> struct Dots<float> {
   u64 s[4], l[4];
-  unsigned e[4];             // bits of M
-  // bits of the power of two in (x, 2 x], at least 2^-100
-  static __device__ __forceinline__ unsigned bound(float x) {
-    const float y = fminf(fmaxf(x, 0x1p-101f), 0x1p122f);
-    return (__float_as_uint(y) & 0x7f800000u) + 0x00800000u;
-  }
-  static __device__ __forceinline__ float warp_max(float x) {     // (x >= 0: its bits compare as integers)
-    return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(x)));
-  }
-  // largest |r|, |p| and |q| of the thread
-  __device__ __forceinline__ void begin(float mr, float mp, float mq) {
-    mr = warp_max(mr);
-    mp = warp_max(mp);
-    mq = warp_max(mq);
-    // up to 16 products per accumulator, half of M to either side (34: room for their rounding)
-    e[0] = bound(34.0f * mr * mr);
-    e[1] = bound(34.0f * mp * mq);
-    e[2] = bound(34.0f * mr * mq);
-    e[3] = bound(34.0f * mq * mq);
+  __device__ __forceinline__ void zero() {
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      s[k] = VT<float>::bcast(__uint_as_float(e[k] | 0x00400000u));
-      l[k] = 0ull;
-    }
+    for (int k = 0; k < 4; ++k) s[k] = l[k] = 0ull;
   }
-  __device__ __forceinline__ void add(int k, u64 x, u64 y) {
-    const u64 t = vfma(x, y, s[k]);
-    const u64 z = vsub(s[k], t);        // -(t - s)
-    l[k] = vadd(l[k], vfma(x, y, z));
+  // sum k of (x, y), with ny = -y
+  __device__ __forceinline__ void add(int k, u64 x, u64 y, u64 ny) {
+    const u64 np = vmul(x, ny);             // -p
+    const u64 e = vfma(x, y, np);           // p + e = x y exactly
+    const u64 t = vsub(s[k], np);
+    const u64 bb = vsub(t, s[k]);
+    const u64 err = vsub(vsub(s[k], vsub(t, bb)), vadd(np, bb));
     s[k] = t;
+    l[k] = vadd(l[k], vadd(err, e));
   }
-  static __device__ __forceinline__ FF plus(FF a, FF b) { return ff_add(a, b); }
+  __device__ __forceinline__ void add_row(u64 r, u64 p, u64 q) {
+    const u64 nr = vsub(0ull, r), nq = vsub(0ull, q);
+    add(0, r, r, nr);
+    add(1, p, q, nq);
+    add(2, r, q, nq);
+    add(3, q, q, nq);
+  }
   static __device__ __forceinline__ FF shfl(FF a, int o) {
     return FF{__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o)};
   }
   static __device__ __forceinline__ double value(FF a) { return (double)a.hi + (double)a.lo; }
-  // the four sums over the warp: lane k returns sum k (k < 4)
+  // ff_add of two pairs of sums at once
+  struct F2 { u64 hi, lo; };
+  static __device__ __forceinline__ F2 plus(F2 a, F2 b) {
+    const u64 t = vadd(a.hi, b.hi), bb = vsub(t, a.hi);
+    const u64 err = vadd(vadd(vsub(a.hi, vsub(t, bb)), vsub(b.hi, bb)), vadd(a.lo, b.lo));
+    const u64 h = vadd(t, err);
+    return F2{h, vsub(err, vsub(h, t))};
+  }
+  // both halves of sums k and k + 1
+  __device__ __forceinline__ F2 halves(int k) const {
+    float a[2], b[2], c[2], d[2];
+    VT<float>::split(s[k], a);
+    VT<float>::split(s[k + 1], b);
+    VT<float>::split(l[k], c);
+    VT<float>::split(l[k + 1], d);
+    const float h0[2] = {a[0], b[0]}, h1[2] = {a[1], b[1]}, l0[2] = {c[0], d[0]}, l1[2] = {c[1], d[1]};
+    return plus(F2{VT<float>::make(h0), VT<float>::make(l0)}, F2{VT<float>::make(h1), VT<float>::make(l1)});
+  }
+  // the four sums over the warp: lane k returns sum k (k < 4); each exchange step halves the
+  // number of sums a lane carries
   __device__ __forceinline__ double warp_sums(int lane) const {
-    int hi = 0, lo = 0;
-    unsigned ek = e[0];
-    bool bad = false;
+    const bool up = lane & 16, up8 = lane & 8;
+    const F2 a = halves(0), b = halves(2), keep = up ? b : a, give = up ? a : b;
+    const F2 f = plus(keep, F2{__shfl_xor_sync(0xffffffffu, give.hi, 16), __shfl_xor_sync(0xffffffffu, give.lo, 16)});
+    float h[2], w[2];
+    VT<float>::split(f.hi, h);
+    VT<float>::split(f.lo, w);
+    FF c = ff_add(up8 ? FF{h[1], w[1]} : FF{h[0], w[0]}, shfl(up8 ? FF{h[0], w[0]} : FF{h[1], w[1]}, 8));
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      float c[2], d[2];
-      VT<float>::split(s[k], c);
-      VT<float>::split(l[k], d);
-      const unsigned b0 = __float_as_uint(c[0]), b1 = __float_as_uint(c[1]);
-      bad |= ((b0 ^ e[k]) & 0xff800000u) != 0 || ((b1 ^ e[k]) & 0xff800000u) != 0;
-      const float iu = __uint_as_float((277u << 23) - e[k]);           // 1 / u = 2^23 / M
-      const int h1 = __reduce_add_sync(0xffffffffu, (int)(b0 + b1 - 2u * (e[k] | 0x00400000u)));
-      const int l1 = __reduce_add_sync(0xffffffffu, __float2int_rn((d[0] + d[1]) * iu * 0x1p20f));
-      if (lane == k) {
-        hi = h1;
-        lo = l1;
-        ek = e[k];
-      }
-    }
-    if (__any_sync(0xffffffffu, bad)) return __longlong_as_double(0x7ff8000000000000ll);
-    // (hi 2^20 + lo) 2^-43 M
-    const double m = __longlong_as_double((long long)(unsigned long long)((ek >> 23) + 896u - 43u) << 52);
-    return (double)((long long)hi * (1 << 20) + lo) * m;
+    for (int o = 4; o > 0; o >>= 1) c = ff_add(c, shfl(c, o));
+    return __shfl_sync(0xffffffffu, value(c), (lane & 3) * 8);
   }
 };
 template <> struct Dots<double> {
   double s[4];
-  __device__ __forceinline__ void begin(double, double, double) { s[0] = s[1] = s[2] = s[3] = 0.0; }
-  __device__ __forceinline__ void add(int k, double x, double y) { s[k] = fma(x, y, s[k]); }
+  __device__ __forceinline__ void zero() { s[0] = s[1] = s[2] = s[3] = 0.0; }
+  __device__ __forceinline__ void add_row(double r, double p, double q) {
+    s[0] = fma(r, r, s[0]);
+    s[1] = fma(p, q, s[1]);
+    s[2] = fma(r, q, s[2]);
+    s[3] = fma(q, q, s[3]);
+  }
   // each exchange step halves the number of sums a lane carries: 6 additions per lane, not 20
   __device__ __forceinline__ double warp_sums(int lane) const {
     const bool up = lane & 16, up8 = lane & 8;
@@ -716,7 +711,6 @@ __global__ void __launch_bounds__(RNT, 2) k_cg_resident(ResArgs<T> g) {
 
       // ---- r -= alpha q, x += alpha p, p = r + beta p, on the block and its halo
       const T al = s_alpha, be = s_beta;
-      T mr = T(0), mp = T(0);
       if (act) {
         const V nal = X::bcast(-al), val = X::bcast(al), vbe = X::bcast(be);
         const T pbody = kb >= 0 ? s_pb[kb] : T(0);
@@ -738,15 +732,6 @@ __global__ void __launch_bounds__(RNT, 2) k_cg_resident(ResArgs<T> g) {
               pn = X::make(c);
             }
             P2[p0 + a * PITCH] = pn;
-            if (REG) {
-              T d[H];
-              X::split(rn, d);
-#pragma unroll
-              for (int h = 0; h < H; ++h) {
-                mr = fmaxf(mr, fabsf(d[h]));
-                mp = fmaxf(mp, fabsf(c[h]));
-              }
-            }
             if (a == 0) {
               if (H == 2) Pt[plast * H] = c[H - 1];
               if (above) Pt[(plast - pw) * H + H - 1] = c[0];
@@ -787,7 +772,6 @@ __global__ void __launch_bounds__(RNT, 2) k_cg_resident(ResArgs<T> g) {
       __syncthreads();
 
       // ---- q = A p and the dot products
-      T mq = T(0);
       BodySum<T> yb;                       // the thread's rows of A p at the nodes of body kb
       if (act) {
         V yl = V(0);                       // q of the last row
@@ -809,10 +793,6 @@ __global__ void __launch_bounds__(RNT, 2) k_cg_resident(ResArgs<T> g) {
           }
           if (REG) q[REG ? a : 0] = y;
           else Q2[a * RNT + tid] = y;
-          if (REG) {
-#pragma unroll
-            for (int h = 0; h < H; ++h) mq = fmaxf(mq, fabsf(c[h]));
-          }
           if (ec) {
 #pragma unroll
             for (int h = 0; h < H; ++h) qe[ecol_at + h * ha + a] = c[h];
@@ -916,16 +896,12 @@ __global__ void __launch_bounds__(RNT, 2) k_cg_resident(ResArgs<T> g) {
 
       // ---- dot products: threads, warps, then the CTA
       Dots<T> d;
-      d.begin(mr, mp, mq);
+      d.zero();
       if (act) {
 #pragma unroll UNR
         for (int a = 0; a < (REG ? ROWS : ha); ++a) {
           if (a < ha) {
-            const V rr = R2[a * RNT + tid], pp = P2[p0 + a * PITCH], qq = REG ? q[REG ? a : 0] : Q2[a * RNT + tid];
-            d.add(0, rr, rr);
-            d.add(1, pp, qq);
-            d.add(2, rr, qq);
-            d.add(3, qq, qq);
+            d.add_row(R2[a * RNT + tid], P2[p0 + a * PITCH], REG ? q[REG ? a : 0] : Q2[a * RNT + tid]);
           }
         }
       }
