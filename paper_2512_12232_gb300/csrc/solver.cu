@@ -2156,8 +2156,10 @@ pf_status solve_core(Batch& b, double U, const pf_solve_opts& o, double* dev_psi
     }
   }
   // k_max == 0 (internal use): only the initial residual, which measures ||b||
-  if (resident) chunk = o.chunk > 0 ? o.chunk : RESIDENT_ITERS;
   const long long max_chunks = o.k_max == 0 ? 0 : o.k_max / chunk + 1000;
+  // (a resident launch ends with the inner solve, so as many of them are allowed as there are
+  // chunks of the streaming kernel: each of those held one restart, too)
+  if (resident && o.chunk <= 0) chunk = RESIDENT_ITERS;
   // Chunks are queued two ahead of the host: slot k holds events (start, after the CG
   // graph, after the refinement kernels) and the pinned poll words / variant states
   // copied after it.  The host retires a slot by waiting on its last event.

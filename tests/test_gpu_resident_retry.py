@@ -30,3 +30,18 @@ def test_solve_after_a_wait_that_gave_up(prec, after):
             assert again.status == 0 and again.info[0]["iters"] == first.info[0]["iters"]
             assert np.array_equal(again.psi.cpu().numpy(), first.psi.cpu().numpy())
             assert np.array_equal(again.body_psi, first.body_psi)
+
+
+def test_restarts_are_bounded_as_in_chunks():
+    """A mixed solve whose tolerance cannot be met restarts until its launches are used up: as many
+    as the streaming kernel's chunks of 256 iterations, k_max / 256 + 1000, and the last ones a
+    launch is queued ahead."""
+    from paper_2512_12232_gb300 import api
+    D = W.BC_DIRICHLET_UY
+    c = W.Case(-4.0, 4.0, -2.0, 2.0, 40, 20, np.array([[0.13, 0.07, 0.6]]), 8, (D, D, D, D))
+    k_max = 300_000
+    with api.mesh_build(c.grid, c.bodies, c.sweeps, c.bc) as g:
+        res = api.psi_solve(g, U=1.0, tol=1e-30, precision=api.PF_MIXED, inner_tol=0.9999, k_max=k_max,
+                            raise_on_failure=False)
+    assert res.info[0]["status"] == 3 and res.info[0]["iters"] < k_max
+    assert res.info[0]["refinements"] >= k_max // 256 + 1000 - 2
