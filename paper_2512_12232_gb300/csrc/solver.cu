@@ -1304,7 +1304,17 @@ __global__ void __launch_bounds__(NT, 4) k_apply_direct(MeshDev m, const int2* _
 #pragma unroll
       for (int u = 0; u < STRIP; ++u) {
         const T dp = win[u + 2][1] - win[u + 1][1];
-        yc[u * row] = fma(kr[1], S[u] + S[u + 2], fma(c2, dp - dm, c1 * S[u + 1]));
+        T out = fma(kr[1], S[u] + S[u + 2], fma(c2, dp - dm, c1 * S[u + 1]));
+        // an infinite value above or below enters two terms of opposite sign here, and a sum of two
+        // finite differences can leave the range: such rows are formed as k_apply forms them
+        if ((__double2hiint((double)out) & 0x7ff00000) == 0x7ff00000) {
+          const T(*w)[FW] = ps + r0 + u;
+          const T nbh[3][3] = {{w[0][col], w[0][col + 1], w[0][col + 2]},
+                               {w[1][col], w[1][col + 1], w[1][col + 2]},
+                               {w[2][col], w[2][col + 1], w[2][col + 2]}};
+          out = q4_row_rect<T>(nbh, krect<T>(V));
+        }
+        yc[u * row] = out;
         dm = dp;
       }
     } else {
