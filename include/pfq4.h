@@ -363,14 +363,23 @@ pf_status pf_apply_timing(pf_batch* b, int precision, int reps, double* us_per_a
 /* Device-event timing of the last pf_psi_solve on this handle. */
 pf_status pf_last_timing(const pf_batch* b, pf_timing* out);
 
-/* Test hook for failure detection without a GPU fault.  With enable = 1, every fused CG
-   launch of later solves on this handle has CTA 0 skip the copies of its first tile and
-   caps each mbarrier wait at 1024 polls, so the consumer warps' bounded wait on that
-   stage gives up: the kernel records the failure in a device flag, drains the copies it
-   did issue, returns, and the solve returns PF_ETIMEOUT.  No wait is unbounded, nothing
-   faults and the CUDA context stays usable.  The handle's iterate is then undefined:
-   destroy it.  enable = 0 restores normal launches.  PF_EINVAL for a NULL handle. */
+/* Test hook for failure detection without a GPU fault.  With enable = 1, a wait of later
+   unpreconditioned solves on this handle gives up after 1024 polls.  Batches whose CG state
+   stays on the chip: the first block of each variant withholds its partial sums of a launch's
+   first iteration, and the blocks' waits for them give up; the kernel records the failure in
+   a device flag and returns.  Other batches: CTA 0 of every fused CG launch skips the copies
+   of its first tile, the consumer warps' wait on that stage gives up, and the kernel records
+   the failure, drains the copies it did issue and returns.  Either way the solve returns
+   PF_ETIMEOUT, no wait is unbounded, nothing faults and the CUDA context stays usable.  The
+   handle's iterate is then undefined; a later solve without warm_start starts afresh.
+   enable = 0 restores normal launches.  PF_EINVAL for a NULL handle. */
 pf_status pf_test_wait_timeout(pf_batch* b, int enable);
+
+/* Test hook: with enable = 1, later unpreconditioned solves on this handle (its
+   velocity-potential and Schur sub-solves included) run the kernel that streams the CG state
+   through memory, also where the batch is small enough for its state to stay on the chip.
+   enable = 0 restores the choice by size.  PF_EINVAL for a NULL handle. */
+pf_status pf_test_streaming(pf_batch* b, int enable);
 
 /* Velocity potential phi of every variant (section "Governing Equation": u = grad phi,
    nabla^2 phi = 0; the contour lines of phi and psi form the flow net).  The same Q4

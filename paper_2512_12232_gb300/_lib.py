@@ -85,6 +85,7 @@ _SIGS = {
     "pf_phi_solve": (C.c_int, [P, C.c_double, C.POINTER(pf_solve_opts), P, P, P]),
     "pf_phi_velocity_field": (C.c_int, [P, C.c_int, P, P, P]),
     "pf_test_wait_timeout": (C.c_int, [P, C.c_int]),
+    "pf_test_streaming": (C.c_int, [P, C.c_int]),
     "pf_apply_timing": (C.c_int, [P, C.c_int, C.c_int, C.POINTER(C.c_double), C.POINTER(C.c_double), P]),
     "pf_last_timing": (C.c_int, [P, C.POINTER(pf_timing)]),
     "pf_surface_velocity": (C.c_int, [P, C.c_int, C.c_int, P, P, C.c_int, C.POINTER(C.c_int), P]),

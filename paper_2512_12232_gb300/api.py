@@ -238,6 +238,10 @@ class Mesh:
         """Test hook: later solves make a bounded device wait give up (PF_ETIMEOUT)."""
         check(L.load().pf_test_wait_timeout(self.handle, int(bool(enable))))
 
+    def test_streaming(self, enable=True):
+        """Test hook: later solves run the streaming CG kernel also where the state fits the chip."""
+        check(L.load().pf_test_streaming(self.handle, int(bool(enable))))
+
 
 def mesh_build(grid, bodies, sweeps, bc=(0, 0, 0, 0), polygons=None) -> Mesh:
     """One variant: grid = (x0, x1, y0, y1, nx, ny), bodies = rows of (cx, cy, r), then the

@@ -418,6 +418,14 @@ pf_status pf_test_wait_timeout(pf_batch* h, int enable) {
   });
 }
 
+pf_status pf_test_streaming(pf_batch* h, int enable) {
+  return guarded([&]() -> pf_status {
+    if (!h) throw Error{PF_EINVAL, "NULL handle"};
+    ((Batch*)h)->test_stream = enable != 0;
+    return PF_OK;
+  });
+}
+
 pf_status pf_last_timing(const pf_batch* h, pf_timing* out) {
   return guarded([&]() -> pf_status {
     const Batch* b = (const Batch*)h;

@@ -143,6 +143,7 @@ pf_status phi_solve(Batch& b, double U, const pf_solve_opts& o, double* dev_phi,
     throw Error{PF_EINVAL, "pf_phi_solve: phi differs between the split copies of a node, one unknown per node cannot hold it"};
   if (o.k_max < 1) throw Error{PF_EINVAL, "k_max must be >= 1"};
   Batch& p = phi_view(b);
+  p.test_stream = b.test_stream;
   p.rhs_active = false;
   p.fixed_bodies = false;
   p.Uv_active = false;

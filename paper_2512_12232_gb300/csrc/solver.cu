@@ -2129,7 +2129,7 @@ pf_status solve_core(Batch& b, double U, const pf_solve_opts& o, double* dev_psi
     if (hdone[1]) throw Error{PF_ETIMEOUT, "a bounded wait in the CG kernel gave up (TMA tile not delivered)"};
     return (double)ms / n;
   };
-  const bool resident = !pcg && o.k_max > 0 && resident_ready(b, prec);
+  const bool resident = !pcg && o.k_max > 0 && !b.test_stream && resident_ready(b, prec);
   const bool tune = b.cg_tune && o.k_max > 0 && !getenv("PFQ4_CG_STAGES") && !pcg && !resident;
   if (tune && !b.stages_tuned[prec]) {
     double best = 1e300;
