@@ -28,6 +28,7 @@ struct Error {                 // thrown inside the library, converted to pf_sta
 
 struct CgConfig {                  // persistent grid + schedule of one fused-CG kernel instance
   bool ready = false;
+  bool open = false;                 // a solve has launched and not come to its end: arrivals may be left in sc.counter
   int G = 0;
   int smem = 0;
   Sched sc{};

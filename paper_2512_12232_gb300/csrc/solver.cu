@@ -2129,6 +2129,11 @@ pf_status solve_core(Batch& b, double U, const pf_solve_opts& o, double* dev_psi
     if (hdone[1]) throw Error{PF_ETIMEOUT, "a bounded wait in the CG kernel gave up (TMA tile not delivered)"};
     return (double)ms / n;
   };
+  // The arrival counters are zero after every whole launch; a CTA whose wait gave up did not arrive.
+  auto use = [&](CgConfig& c) {
+    if (c.open) PF_CUDA(cudaMemsetAsync(c.sc.counter, 0, b.nv * sizeof(int), s));
+    c.open = true;
+  };
   const bool resident = !pcg && o.k_max > 0 && !b.test_stream && resident_ready(b, prec);
   const bool tune = b.cg_tune && o.k_max > 0 && !getenv("PFQ4_CG_STAGES") && !pcg && !resident;
   if (tune && !b.stages_tuned[prec]) {
@@ -2137,6 +2142,7 @@ pf_status solve_core(Batch& b, double U, const pf_solve_opts& o, double* dev_psi
     for (int ns = 2; ns <= 4; ++ns) {
       b.cg_stages = ns;
       CgConfig& c = cg_config(b, prec, ns);
+      use(c);
       c.active.assign(b.nv, 1);
       cg_sched_write(b, c);
       const double per = timed_launches(CG_TUNE_LAUNCHES, false);
@@ -2149,6 +2155,7 @@ pf_status solve_core(Batch& b, double U, const pf_solve_opts& o, double* dev_psi
   cudaGraphExec_t ex = resident ? nullptr : pcg ? get_pcg_graph(b, chunk) : get_graph(b, prec, chunk);
   CgConfig none;
   CgConfig& cc = resident ? none : cg_config(b, prec, b.cg_stages);
+  if (!pcg && !resident) use(cc);
   if (!pcg && !resident &&
       (cc.active.size() != (size_t)b.nv || std::find(cc.active.begin(), cc.active.end(), 0) != cc.active.end())) {
     cc.active.assign(b.nv, 1);                   // a solve starts with every variant running
@@ -2246,6 +2253,7 @@ pf_status solve_core(Batch& b, double U, const pf_solve_opts& o, double* dev_psi
   PF_CUDA(cudaMemcpyAsync(fin.data(), b.state, b.nv * sizeof(VarState), cudaMemcpyDeviceToHost, s));
   PF_CUDA(cudaStreamSynchronize(s));
   if (resident) end_resident(b, prec);
+  else if (!pcg) for (CgConfig& c : b.cg_cfg[prec]) c.open = false;
   float tot = 0;
   PF_CUDA(cudaEventElapsedTime(&tot, b.ev[3], b.ev[4]));
   b.solved = true;

@@ -56,3 +56,17 @@ def test_which_kernel_ran(api, prec):
             assert (n % 256 == 0 and n >= it) if on else n == it
             assert it % 256                     # (else the counts would not tell the kernels apart)
             assert res.info[0]["rel_true_residual"] <= 1e-8 and np.all(np.isfinite(res.body_psi))
+
+
+def test_bounded_wait_of_the_streaming_kernel(api):
+    """The wait that gives up is the one for a tile's copy, and a later solve on the handle is whole."""
+    from paper_2512_12232_gb300 import _lib
+    c = W.five_cylinder_case(0.5, 256, 128, 20)
+    with api.mesh_build(c.grid, c.bodies, c.sweeps, c.bc) as g:
+        first = api.psi_solve(g, U=1.0, tol=1e-8, precision=api.PF_MIXED)
+        g.test_wait_timeout(True)
+        with pytest.raises(_lib.PfError, match="TMA tile"):
+            api.psi_solve(g, U=2.0, tol=1e-8, precision=api.PF_MIXED, chunk=4)
+        g.test_wait_timeout(False)
+        again = api.psi_solve(g, U=1.0, tol=1e-8, precision=api.PF_MIXED)
+        assert np.array_equal(again.psi.cpu().numpy(), first.psi.cpu().numpy())
