@@ -6,9 +6,15 @@
 //   * free unknowns: one V(1,1)-cycle of geometric multigrid on the logical node grid of
 //     each variant.  Level 0 is the mesh itself with its Q4 element matrices (the FP32
 //     operator of the CG); level l+1 has ceil(n_l / 2) cells per direction, coarse node I
-//     sitting on fine node min(2I, n_l).  Interpolation P is bilinear along the index
-//     lines (an odd fine node takes half of each coarse neighbour, the last node of an odd
-//     line copies its coarse node).  A coarse node carries an unknown only if the fine node
+//     sitting on fine node min(2I, n_l), except towards a natural side, where an odd n_l is
+//     halved downwards: the last fine line would otherwise be a coarse line one fine cell from
+//     its neighbour, at every level again, until the two are 2^l times closer than the others.
+//     The damped sweep amplifies the difference of such a pair (the last eigenvalue of D^-1 A
+//     is 3 there, and 3 omega > 2), so M is not positive definite and the CG stagnates (257
+//     cells to a natural outlet).  At a Dirichlet side the last line carries no unknown.
+//     Interpolation P is bilinear along the index lines (an odd fine node takes half of each
+//     coarse neighbour, the last node of an odd line copies its coarse node, or the last coarse
+//     one where the line was halved downwards).  A coarse node carries an unknown only if the fine node
 //     under it does (constraints are injected), and P has no entries for constrained
 //     nodes.  Coarse operators are Galerkin products A_{l+1} = P^T A_l P (9-point
 //     stencils, formed once in FP32, the precision the cycle applies them in).  Smoother: damped Jacobi (omega = 0.85), one sweep
@@ -51,29 +57,29 @@ constexpr int MG_COARSE_SWEEPS = 100;    // Jacobi sweeps of the coarsest solve
 constexpr int MG_MAXC = 17 * 17;         // nodes of a coarsest level at most
 
 // ---------------------------------------------------------------- index rules
-// Weight of coarse index I in the interpolation of fine index i on a line of n cells.
-__device__ __forceinline__ double pw(int i, int n, int I) {
+// Weight of coarse index I in the interpolation of fine index i on a line of n cells, nc coarse ones.
+__device__ __forceinline__ double pw(int i, int n, int nc, int I) {
   if ((i & 1) == 0) return I == (i >> 1) ? 1.0 : 0.0;
-  if (i == n) return I == ((i + 1) >> 1) ? 1.0 : 0.0;
+  if (i == n) return I == min((i + 1) >> 1, nc) ? 1.0 : 0.0;
   return (I == ((i - 1) >> 1) || I == ((i + 1) >> 1)) ? 0.5 : 0.0;
 }
 // Coarse parents of fine index i: count, indices and weights.
-__device__ __forceinline__ int parents(int i, int n, int* I, double* w) {
+__device__ __forceinline__ int parents(int i, int n, int nc, int* I, double* w) {
   if ((i & 1) == 0) { I[0] = i >> 1; w[0] = 1.0; return 1; }
-  if (i == n) { I[0] = (i + 1) >> 1; w[0] = 1.0; return 1; }
+  if (i == n) { I[0] = min((i + 1) >> 1, nc); w[0] = 1.0; return 1; }
   I[0] = (i - 1) >> 1; I[1] = (i + 1) >> 1; w[0] = w[1] = 0.5;
   return 2;
 }
 __device__ __forceinline__ int fine_of(int I, int n) { return min(2 * I, n); }
 // The same rules in FP32 for the cycle (the weights 1 and 1/2 are exact in FP32).
-__device__ __forceinline__ float pwf(int i, int n, int I) {
+__device__ __forceinline__ float pwf(int i, int n, int nc, int I) {
   if ((i & 1) == 0) return I == (i >> 1) ? 1.0f : 0.0f;
-  if (i == n) return I == ((i + 1) >> 1) ? 1.0f : 0.0f;
+  if (i == n) return I == min((i + 1) >> 1, nc) ? 1.0f : 0.0f;
   return (I == ((i - 1) >> 1) || I == ((i + 1) >> 1)) ? 0.5f : 0.0f;
 }
-__device__ __forceinline__ int parentsf(int i, int n, int* I, float* w) {
+__device__ __forceinline__ int parentsf(int i, int n, int nc, int* I, float* w) {
   if ((i & 1) == 0) { I[0] = i >> 1; w[0] = 1.0f; return 1; }
-  if (i == n) { I[0] = (i + 1) >> 1; w[0] = 1.0f; return 1; }
+  if (i == n) { I[0] = min((i + 1) >> 1, nc); w[0] = 1.0f; return 1; }
   I[0] = (i - 1) >> 1; I[1] = (i + 1) >> 1; w[0] = w[1] = 0.5f;
   return 2;
 }
@@ -224,11 +230,11 @@ __global__ void k_mg_rap(LvArgs c, float* A32c, float* dinvc, MeshDev m, const u
     // the entry scaled by 2^-h (h halves): exact, one FP32 multiply by that power of two
     for (int ay = fy - 1; ay <= fy + 1; ++ay) {
       if (ay < 0 || ay > df.y) continue;
-      const double wy = pw(ay, df.y, q.j);
+      const double wy = pw(ay, df.y, q.ny, q.j);
       if (wy == 0.0) continue;
       for (int ax = fx - 1; ax <= fx + 1; ++ax) {
         if (ax < 0 || ax > df.x) continue;
-        const double wxa = pw(ax, df.x, q.i);
+        const double wxa = pw(ax, df.x, q.nx, q.i);
         const int ha = (wxa == 0.5) + (wy == 0.5);       // halves of wa = wxa * wy
         if (wxa == 0.0 || !factive(ax, ay)) continue;
         float st[9];
@@ -243,7 +249,7 @@ __global__ void k_mg_rap(LvArgs c, float* A32c, float* dinvc, MeshDev m, const u
             if (sv == 0.0f || bx < 0 || by < 0 || bx > df.x || by > df.y || !factive(bx, by)) continue;
             int Ix[2], Iy[2];
             double wx[2], wyb[2];
-            const int nxp = parents(bx, df.x, Ix, wx), nyp = parents(by, df.y, Iy, wyb);
+            const int nxp = parents(bx, df.x, q.nx, Ix, wx), nyp = parents(by, df.y, q.ny, Iy, wyb);
             for (int u = 0; u < nyp; ++u)
               for (int t = 0; t < nxp; ++t) {
                 const int ddx = Ix[t] - q.i, ddy = Iy[u] - q.j;
@@ -345,7 +351,7 @@ __device__ __forceinline__ float coarse_interp(const FineArgs& a, int v, const D
   const long long oc = a.c_off[v];
   int Ix[2], Iy[2];
   float wx[2], wy[2];
-  const int nxp = parentsf(i, V.nx, Ix, wx), nyp = parentsf(j, V.ny, Iy, wy);
+  const int nxp = parentsf(i, V.nx, dc.x, Ix, wx), nyp = parentsf(j, V.ny, dc.y, Iy, wy);
   float e = 0.0f;
   for (int u = 0; u < nyp; ++u)
     for (int t = 0; t < nxp; ++t) e += wx[t] * wy[u] * a.c_zb[oc + (long long)Iy[u] * (dc.x + 1) + Ix[t]];
@@ -891,11 +897,11 @@ __global__ void __launch_bounds__(256) k_mg_restrict(LvArgs c, int lc, const int
 #pragma unroll
     for (int dy = -1; dy <= 1; ++dy) {
       const int ay = fy + dy;
-      const float wy = (ay < 0 || ay > df.y) ? 0.0f : pwf(ay, df.y, q.j);
+      const float wy = (ay < 0 || ay > df.y) ? 0.0f : pwf(ay, df.y, q.ny, q.j);
 #pragma unroll
       for (int dx = -1; dx <= 1; ++dx) {
         const int ax = fx + dx;
-        const float w = (ax < 0 || ax > df.x) ? 0.0f : pwf(ax, df.x, q.i) * wy;
+        const float w = (ax < 0 || ax > df.x) ? 0.0f : pwf(ax, df.x, q.nx, q.i) * wy;
         if (w == 0.0f) continue;
         const long long na = fine0 ? V.base + (long long)ay * V.P + ax : of + (long long)ay * (df.x + 1) + ax;
         s += w * res_f[na];     // res is zero at every node without an unknown
@@ -960,7 +966,7 @@ __global__ void __launch_bounds__(256) k_mg_prolong(LvArgs f, LvArgs c, int l, c
   } else {
     int Ix[2], Iy[2];
     float wx[2], wy[2];
-    const int nxp = parentsf(q.i, q.nx, Ix, wx), nyp = parentsf(q.j, q.ny, Iy, wy);
+    const int nxp = parentsf(q.i, q.nx, dc.x, Ix, wx), nyp = parentsf(q.j, q.ny, dc.y, Iy, wy);
     for (int u = 0; u < nyp; ++u)
       for (int t = 0; t < nxp; ++t) e += wx[t] * wy[u] * c.zb[oc + (long long)Iy[u] * (dc.x + 1) + Ix[t]];
   }
@@ -1281,7 +1287,11 @@ void mg_setup(Batch& b) {
 
 // Level counts and the packed layout of every coarse level, allocated once per handle.
 static void mg_layout(Batch& b) {
-  // levels per variant: coarsen while a level has more than MG_CMAX cells in a direction
+  // levels per variant: coarsen while a level has more than MG_CMAX cells in a direction.  (The
+  // velocity potential is given at x = x0 and x1 and has natural conditions on the other sides.)
+  const bool natural_right = !b.dirichlet_x && b.bc[1] == PF_BC_NATURAL;
+  const bool natural_top = b.dirichlet_x || b.bc[3] == PF_BC_NATURAL;
+  auto coarse_cells = [](int n, bool natural) { return natural && n > 1 ? n / 2 : (n + 1) / 2; };
   b.mg_Lv.assign(b.nv, 1);
   std::vector<std::vector<int2>> dims(b.nv);
   int L = 1;
@@ -1289,8 +1299,8 @@ static void mg_layout(Batch& b) {
     int nx = b.hv[v].g.nx, ny = b.hv[v].g.ny;
     dims[v].push_back(make_int2(nx, ny));
     do {
-      nx = (nx + 1) / 2;
-      ny = (ny + 1) / 2;
+      nx = coarse_cells(nx, natural_right);
+      ny = coarse_cells(ny, natural_top);
       dims[v].push_back(make_int2(nx, ny));
     } while (std::max(nx, ny) > MG_CMAX);
     b.mg_Lv[v] = (int)dims[v].size();
