@@ -130,7 +130,8 @@ typedef struct pf_solve_opts {
                               that every CTA's measured time evens out (kept for later solves).
                               This changes the order in which the dot products are summed:
                               results agree with an untuned solve to rounding, not bit for bit.
-                              0: schedule from the static per-tile cost estimate (deterministic). */
+                              0: schedule from the static per-tile cost estimate (deterministic).
+                              No effect where the CG state stays on the chip (no schedule there) */
     int criterion;         /* PF_TOL_REL_TRUE (0) or PF_TOL_PAPER_ABS (1); any other value: PF_EINVAL */
     int preconditioner;    /* PF_PRECOND_NONE (0): the paper's CG; PF_PRECOND_MG (1): CG preconditioned by a
                               geometric multigrid V-cycle (PF_MIXED only); any other value: PF_EINVAL */
@@ -152,9 +153,12 @@ typedef struct pf_timing {
     long long residual_launches;
     double solve_ms;             /* device time of the whole solve, events on the call's stream */
     double cg_bytes_per_launch;  /* algorithmic HBM bytes of one fused CG launch, averaged over the
-                                    launches of the solve (variants already converged move nothing) */
+                                    launches of the solve (variants already converged move nothing);
+                                    where the CG state stays on the chip, the state's way in and out,
+                                    once per inner solve, spread over the iterations */
     long long kernel_launches;   /* kernels launched by this handle since it was built (mesh + solves) */
-    int cg_stages;               /* pipeline depth of the fused CG kernel in the last solve (2..4) */
+    int cg_stages;               /* pipeline depth of the fused CG kernel in the last solve (2..4; the
+                                    depth it would have where the CG state stays on the chip) */
 } pf_timing;
 
 typedef struct pf_batch pf_batch;   /* opaque: one or more mesh variants and their solver state */

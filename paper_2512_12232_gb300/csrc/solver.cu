@@ -2273,8 +2273,15 @@ pf_status solve_core(Batch& b, double U, const pf_solve_opts& o, double* dev_psi
     // coefficient bytes: the cells whose stored K_e the operator of this precision reads
     const long long n_gen = prec == PF_MIXED ? b.hv[v].n_gen32_cells : M.n_general_cells;
     const double bv = per_node_free * M.n_free + per_body * M.n_body_nodes + 1.0 * M.n_nodes + per_gen * n_gen;
-    if (!pcg) bytes_done += bv * (double)S.iters;
-    if (resident) launches = std::max(launches, S.iters);   // a resident iteration counts as a launch of the streaming kernel
+    if (resident) {
+      // the state records come and go once per inner solve (and per pause), with the tags and the
+      // stored coefficients; iterations move nothing.  An iteration counts as a launch
+      const double moved = per_node_free * M.n_free + 1.0 * M.n_nodes + 48.0 * n_gen;
+      bytes_done += moved * (double)std::max<long long>(std::max(0, S.n_resid - 1), (S.iters + chunk - 1) / chunk);
+      launches = std::max(launches, S.iters);
+    } else if (!pcg) {
+      bytes_done += bv * (double)S.iters;
+    }
     if (info) {
       info[v].iters = S.iters;
       info[v].refinements = std::max(0, S.n_resid - 1);
