@@ -1202,17 +1202,35 @@ struct Cutter {
   int W, R, H;                         // nodes per row, rows, halves of a strip
   int tx = 0, ty = 0;                  // 64 x 16 tiles
   std::vector<uint8_t> stored;         // [ty][tx] some operator row needs stored coefficients
+  std::vector<std::vector<int>> ends;  // [column parts][part][ty] where plain runs end, made when first asked for
 
-  // rows to which tile rows of column part [i0, i0 + w) without stored coefficients run on: 0
-  // where the tile row has stored ones
-  void runs(int i0, int w, std::vector<int>& plain_to) const {
-    const int last = std::min(W - 1, i0 + w - 1);
-    plain_to.assign(ty, 0);
-    for (int t = ty - 1; t >= 0; --t) {
-      bool st = false;
-      for (int c = i0 / CTX; c <= last / CTX && !st; ++c) st = stored[(size_t)t * tx + c] != 0;
-      if (!st) plain_to[t] = t + 1 < ty && plain_to[t + 1] ? plain_to[t + 1] : std::min(R, (t + 1) * CTY);
+  // rows to which tile rows of the column parts of width w without stored coefficients run on: 0
+  // where the tile row has stored ones.  (Kept: every candidate of the search asks for the same.)
+  const int* runs(int nbx, int w) {
+    if ((int)ends.size() <= nbx) ends.resize(nbx + 1);
+    std::vector<int>& e = ends[nbx];
+    if (e.empty()) {
+      e.assign((size_t)nbx * ty, 0);
+      for (int p = 0; p < nbx; ++p) {
+        const int c0 = p * w / CTX, c1 = std::min(W - 1, (p + 1) * w - 1) / CTX;
+        int* const to = e.data() + (size_t)p * ty;
+        for (int t = ty - 1; t >= 0; --t) {
+          bool st = false;
+          for (int c = c0; c <= c1 && !st; ++c) st = stored[(size_t)t * tx + c] != 0;
+          if (!st) to[t] = t + 1 < ty && to[t + 1] ? to[t + 1] : std::min(R, (t + 1) * CTY);
+        }
+      }
     }
+    return e.data();
+  }
+  // Blocks of `threads` threads with at most that many rows of a half strip: no cut has fewer.  A
+  // block without stored rows holds no node of a stored tile.
+  double least(int rows, int grows, int threads) const {
+    double st = 0.0;
+    for (int t = 0; t < ty; ++t)
+      for (int c = 0; c < tx; ++c)
+        if (stored[(size_t)t * tx + c]) st += (double)std::min(CTX, W - c * CTX) * std::min(CTY, R - t * CTY);
+    return (st / std::min(rows, grows) + ((double)W * R - st) / std::max(rows, grows)) / ((double)threads * H);
   }
   struct Part { int i0, w, ns, unit, rows, grows; };
 
@@ -1222,7 +1240,7 @@ struct Cutter {
   // with fewer blocks is taken, `forks` times per column part (once: 16 grids of 257x129 nodes
   // with an airfoil each need 256 blocks in place of 320, so that all of them fit the chip; more
   // often costs host time that doubles with every fork and gains under 2 % of the blocks).
-  int down(const Part& c, const std::vector<int>& plain_to, int j, int forks, double& slots, std::vector<RItem>* out) const {
+  int down(const Part& c, const int* plain_to, int j, int forks, double& slots, std::vector<RItem>* out) const {
     int n = 0;
     while (j < R) {
       const int end = plain_to[j / CTY], left = (R - j + c.unit - 1) / c.unit;
@@ -1262,35 +1280,35 @@ struct Cutter {
     return n;
   }
 
-  // one column part: appends (j0, ha, gen); false if the exchange lists would overflow
-  bool column(int i0, int w, int ns, int rows, int grows, std::vector<RItem>* out, int& parts, double& slots) const {
+  // column part p: appends (j0, ha, gen); false if the exchange lists would overflow
+  bool column(int p, const int* ends_w, int w, int ns, int rows, int grows, std::vector<RItem>* out, int& parts, double& slots) const {
     const int unit = ns * H, fit = (HMAX - 2 * (w + 2)) / (2 * unit);
     if (fit < 2) return false;
-    const Part c{i0, w, ns, unit, std::min(rows, fit), std::min(grows, fit)};
-    std::vector<int> plain_to;
-    runs(i0, w, plain_to);
-    parts += down(c, plain_to, 0, 1, slots, out);
+    const Part c{p * w, w, ns, unit, std::min(rows, fit), std::min(grows, fit)};
+    parts += down(c, ends_w + (size_t)p * ty, 0, 1, slots, out);
     return true;
   }
 
   // the cut with the fewest blocks (ties: fewer rows in all)
-  bool best(int rows, int grows, int threads, std::vector<RItem>& out) const {
+  bool best(int rows, int grows, int threads, std::vector<RItem>& out) {
     double best_cost = 1e300;
-    int bw = 0, bns = 0;
+    int bn = 0, bw = 0, bns = 0;
     for (int nbx = (W + threads - 1) / threads; nbx <= W; ++nbx) {
       const int w = (W + nbx - 1) / nbx;
       if (w < 32 && nbx > 1) break;
       if ((nbx - 1) * w >= W) continue;                // the last column part would be empty
       const int most = std::min(NSMAX, threads / w);
+      const int* const e = runs(nbx, w);
       for (int ns = most; ns >= std::max(1, most - 1); --ns) {
         if (w * ns < threads / 2 && W >= threads) continue;   // half the threads idle
         int parts = 0;
         double slots = 0.0;
         bool ok = true;
-        for (int bx = 0; bx < nbx && ok && parts < best_cost; ++bx) ok = column(bx * w, w, ns, rows, grows, nullptr, parts, slots);
+        for (int bx = 0; bx < nbx && ok && parts < best_cost; ++bx) ok = column(bx, e, w, ns, rows, grows, nullptr, parts, slots);
         const double cost = parts + 0.01 * slots;
         if (ok && cost < best_cost) {
           best_cost = cost;
+          bn = nbx;
           bw = w;
           bns = ns;
         }
@@ -1300,7 +1318,7 @@ struct Cutter {
     if (bw == 0) return false;
     int parts = 0;
     double slots = 0.0;
-    for (int i0 = 0; i0 < W; i0 += bw) column(i0, bw, bns, rows, grows, &out, parts, slots);
+    for (int p = 0; p < bn; ++p) column(p, runs(bn, bw), bw, bns, rows, grows, &out, parts, slots);
     return true;
   }
 };
@@ -1357,6 +1375,9 @@ bool resident_ready(Batch& b, int precision) {
   PF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, f, RNT, R.smem));
   const long long G = (long long)occ * b.nsm;
   if (G < 1) return false;
+  double nodes = 0.0;
+  for (auto& h : b.hv) nodes += (double)(h.g.nx + 1) * (h.g.ny + 1);
+  if (nodes > 2.0 * G * RNT * H * rows) return false;
   // tile flags
   const long long T = b.Tcg;
   std::vector<int2> ij(T);
@@ -1367,7 +1388,6 @@ bool resident_ready(Batch& b, int precision) {
   PF_CUDA(cudaMemcpyAsync(fl.data(), b.tile_cg_gen, T, cudaMemcpyDeviceToHost, b.stream));
   PF_CUDA(cudaStreamSynchronize(b.stream));
   std::vector<Cutter> cut(b.nv);
-  double nodes = 0.0;
   for (int v = 0; v < b.nv; ++v) {
     Cutter& c = cut[v];
     c.W = b.hv[v].g.nx + 1;
@@ -1376,7 +1396,6 @@ bool resident_ready(Batch& b, int precision) {
     c.tx = (c.W + CTX - 1) / CTX;
     c.ty = (c.R + CTY - 1) / CTY;
     c.stored.assign((size_t)c.tx * c.ty, 0);
-    nodes += (double)c.W * c.R;
     if ((double)c.W * c.R > (double)G * RNT * H * rows) return false;
   }
   const uint8_t bit = f64 ? TILE_ROW64 : TILE_ROW32;
@@ -1392,29 +1411,48 @@ bool resident_ready(Batch& b, int precision) {
     }
     return total <= most;
   };
+  auto least = [&](int cap, int gcap, int threads) {
+    double n = 0.0;
+    for (auto& c : cut) n += std::max(1.0, std::ceil(c.least(cap, std::max(2, std::min(grows, gcap)), threads) * (1.0 - 1e-9)));
+    return n;
+  };
   // all at once: the cut whose iteration is estimated shortest.  An iteration's fixed part costs
   // about as much as five rows; a row with stored coefficients 1.6 times (FP64: 1.5 times) a row
-  // without; two blocks on one SM share it
-  double best_cost = 1e300;
-  int best_cap = 0, best_gcap = 0, best_threads = 0;
+  // without; two blocks on one SM share it.  From the least estimate up, as far as one can still
+  // win, and cut only where the least number of blocks leaves room.  A handle's first solve is
+  // longer than its second by 0.95 ms with five 403x201 channels (every candidate in turn: 2.6),
+  // 0.85 with one 1024x512 grid in FP64 (4.4), 0.8 on 6000x60 cells (4.6), and 0.75 where two
+  // 2048x1024 grids do not fit (2.1)
+  struct Candidate { double cost; int threads, cap, gc; };
+  std::vector<Candidate> cand;
   for (int threads : {64, 128, RNT})
     for (int cap = 2; cap <= rows; ++cap)
-      for (int gc = std::max(2, cap / 2); gc <= std::min(cap, grows); ++gc) {
-        if (nodes > (double)G * threads * H * cap) continue;
-        const double cost = (5.0 + std::max((double)cap, (f64 ? 1.5 : 1.6) * gc)) * threads / RNT;
-        if (cost >= best_cost || !plan(cap, gc, threads, G)) continue;
-        const double c2 = cost * (double)((total + b.nsm - 1) / b.nsm);
-        if (c2 < best_cost) {
-          best_cost = c2;
-          best_cap = cap;
-          best_gcap = gc;
-          best_threads = threads;
-        }
-      }
-  const bool spread = best_cap > 0;
-  if (spread) plan(best_cap, best_gcap, best_threads, G);
-  // else the largest blocks, and the variants queue
-  if (!spread && (nodes > 2.0 * G * RNT * H * rows || !plan(rows, grows, RNT, 2 * G))) return false;
+      for (int gc = std::max(2, cap / 2); gc <= std::min(cap, grows); ++gc)
+        if (nodes <= (double)G * threads * H * cap)
+          cand.push_back({(5.0 + std::max((double)cap, (f64 ? 1.5 : 1.6) * gc)) * threads / RNT, threads, cap, gc});
+  std::vector<int> by_cost(cand.size());
+  for (size_t k = 0; k < cand.size(); ++k) by_cost[k] = (int)k;
+  std::stable_sort(by_cost.begin(), by_cost.end(), [&](int x, int y) { return cand[x].cost < cand[y].cost; });
+  double best_cost = 1e300;
+  int best = -1, planned = -1;           // (of two with one cost the first in the loops' order)
+  for (int k : by_cost) {
+    const Candidate& c = cand[k];
+    if (c.cost > best_cost) break;
+    const double n = least(c.cap, c.gc, c.threads), low = c.cost * std::ceil(n / b.nsm);
+    if (n > (double)G || low > best_cost || (low == best_cost && k > best)) continue;
+    planned = k;
+    if (!plan(c.cap, c.gc, c.threads, G)) continue;
+    const double c2 = c.cost * (double)((total + b.nsm - 1) / b.nsm);
+    if (c2 < best_cost || (c2 == best_cost && k < best)) {
+      best_cost = c2;
+      best = k;
+    }
+  }
+  if (best >= 0) {
+    if (planned != best) plan(cand[best].cap, cand[best].gc, cand[best].threads, G);
+  } else if (least(rows, grows, RNT) > 2.0 * G || !plan(rows, grows, RNT, 2 * G)) {
+    return false;                        // else the largest blocks, and the variants queue
+  }
   size_t most = 0;
   for (auto& x : blocks) most = std::max(most, x.size());
   if ((long long)most > G || total > (1 << 24)) return false;
