@@ -47,6 +47,7 @@ struct CgConfig {                  // persistent grid + schedule of one fused-CG
 // How a batch runs with its CG state on the chip (resident.cu), per precision.
 struct ResPlan {
   bool made = false, ok = false;     // the plan was looked for; the batch fits
+  bool queued = false;               // more blocks than the chip holds at once
   bool open = false;                 // a solve has launched and not come to its end: d_pw and d_bc may hold
                                      // words numbered past d_epoch
   size_t smem = 0;                   // dynamic shared memory of a CTA
@@ -280,7 +281,7 @@ void export_psi(Batch& b, double* dev_psi);
 void body_values(Batch& b, std::vector<double>& C);
 
 // resident.cu
-bool resident_ready(Batch& b, int precision);
+bool resident_ready(Batch& b, int precision, int chunk);
 void launch_resident(Batch& b, int precision, int max_it);
 void end_resident(Batch& b, int precision);
 void drop_resident(Batch& b);

@@ -1347,13 +1347,23 @@ void clear_exchange(Batch& b, ResPlan& R) {
 // the shortest iteration; up to twice that, blocks are as large as a CTA holds and the variants
 // queue.  Larger batches, and variants that need more blocks than there are resident CTAs,
 // take the streaming kernel of solver.cu: it is then bound by bytes, no longer by latency.
-bool resident_ready(Batch& b, int precision) {
+static bool make_plan(Batch& b, int precision);
+
+// ... and does it pay with `chunk` iterations a launch (0: as many as the inner solve takes)?  A
+// launch carries the state from and to memory.  Time of the streaming kernel over that of this one,
+// FP32, at chunks of 4, 6, 8, 12, 16: one 1900x951 grid 0.91, 1.07, 1.18, 1.36, 1.46; twenty of
+// 400x200, which queue, 0.63, 0.76, 0.86, 0.98, 1.07.
+bool resident_ready(Batch& b, int precision, int chunk) {
   ResPlan& R = b.res[precision];
-  if (R.made) {
-    // after a solve that was broken off (a wait that gave up) the last numbers in use are not known
-    if (R.ok && R.open) clear_exchange(b, R);
-    return R.ok;
-  }
+  if (!R.made) make_plan(b, precision);
+  if (!R.ok || (chunk > 0 && chunk < (R.queued ? 16 : 6))) return false;
+  // after a solve that was broken off (a wait that gave up) the last numbers in use are not known
+  if (R.open) clear_exchange(b, R);
+  return true;
+}
+
+static bool make_plan(Batch& b, int precision) {
+  ResPlan& R = b.res[precision];
   R.made = true;
   R.ok = false;
   const bool f64 = precision == PF_FP64;
@@ -1462,6 +1472,46 @@ bool resident_ready(Batch& b, int precision) {
   std::stable_sort(ord.begin(), ord.end(), [&](int x, int y) {
     return std::max(b.hv[x].g.nx, b.hv[x].g.ny) > std::max(b.hv[y].g.nx, b.hv[y].g.ny);
   });
+  R.queued = best < 0;
+  if (R.queued && f64) {
+    // In FP64 a full chip gains little over the streaming kernel (both wait for the FP64 pipe), so
+    // a queue has to pack well: few large variants leave CTAs without work (two 842x411 grids, one
+    // after the other, 90 against 57 us an iteration), many small ones do not (63 of 155x66: 32
+    // against 67).  Times of an iteration of the longest variant, fitted to 86 measured batches (5.5
+    // and 9 us rms): with the chip filled `span` times over, and for the streaming kernel, whose
+    // variants drop out as they finish.  At 0.88 none of them is slower here, two in five gain.
+    // (FP32: 69 batches, 0.98 to 2.2 times as fast; no rule.)
+    std::vector<double> tiles(b.nv, 0.0), gen(b.nv, 0.0);
+    for (long long t = 0; t < T; ++t) {
+      tiles[var[t]] += 1.0;
+      if (fl[t] & TILE_GEN64) gen[var[t]] += 1.0;
+    }
+    std::vector<std::pair<double, long long>> run;     // running variants: end, blocks (a heap, earliest first)
+    const auto later = [](const std::pair<double, long long>& x, const std::pair<double, long long>& y) { return x.first > y.first; };
+    double now = 0.0, span = 0.0, area = 0.0, nt = 0.0, ng = 0.0;
+    long long left = G;
+    const double longest = std::max(b.hv[ord[0]].g.nx, b.hv[ord[0]].g.ny);
+    for (int v : ord) {
+      const double w = std::max(b.hv[v].g.nx, b.hv[v].g.ny) / longest;
+      const long long n = (long long)blocks[v].size();
+      while (left < n) {
+        std::pop_heap(run.begin(), run.end(), later);
+        now = run.back().first;
+        left += run.back().second;
+        run.pop_back();
+      }
+      left -= n;
+      run.push_back({now + w, n});
+      std::push_heap(run.begin(), run.end(), later);
+      span = std::max(span, now + w);
+      area += w * (double)n / (double)G;
+      nt += w * tiles[v];
+      ng += w * gen[v];
+    }
+    const double here = (31.0 + 6.0 * ng / nt) * span + 7.5 * area;
+    const double streamed = 31.0 + 0.0385 * nt + 0.0214 * ng + 0.19 * b.nv;
+    if (here > 0.88 * streamed) return false;
+  }
   std::vector<RItem> items;
   std::vector<RVar> vars(b.nv);
   items.reserve(total);

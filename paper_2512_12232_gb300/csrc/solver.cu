@@ -2134,7 +2134,7 @@ pf_status solve_core(Batch& b, double U, const pf_solve_opts& o, double* dev_psi
     if (c.open) PF_CUDA(cudaMemsetAsync(c.sc.counter, 0, b.nv * sizeof(int), s));
     c.open = true;
   };
-  const bool resident = !pcg && o.k_max > 0 && !b.test_stream && resident_ready(b, prec);
+  const bool resident = !pcg && o.k_max > 0 && !b.test_stream && resident_ready(b, prec, o.chunk);
   const bool tune = b.cg_tune && o.k_max > 0 && !getenv("PFQ4_CG_STAGES") && !pcg && !resident;
   if (tune && !b.stages_tuned[prec]) {
     double best = 1e300;
