@@ -12,6 +12,9 @@
 //     The damped sweep amplifies the difference of such a pair (the last eigenvalue of D^-1 A
 //     is 3 there, and 3 omega > 2), so M is not positive definite and the CG stagnates (257
 //     cells to a natural outlet).  At a Dirichlet side the last line carries no unknown.
+//     Between two natural sides the last two lines (one cell) become one: they would otherwise
+//     stay as they are while the other direction is halved on, ever closer in comparison
+//     (4000x40 cells of phi).
 //     Interpolation P is bilinear along the index lines (an odd fine node takes half of each
 //     coarse neighbour, the last node of an odd line copies its coarse node, or the last coarse
 //     one where the line was halved downwards).  A coarse node carries an unknown only if the fine node
@@ -1314,9 +1317,9 @@ void mg_setup(Batch& b) {
 static void mg_layout(Batch& b) {
   // levels per variant: coarsen while a level has more than MG_CMAX cells in a direction.  (The
   // velocity potential is given at x = x0 and x1 and has natural conditions on the other sides.)
-  const bool natural_right = !b.dirichlet_x && b.bc[1] == PF_BC_NATURAL;
-  const bool natural_top = b.dirichlet_x || b.bc[3] == PF_BC_NATURAL;
-  auto coarse_cells = [](int n, bool natural) { return natural && n > 1 ? n / 2 : (n + 1) / 2; };
+  bool natural[4];
+  for (int k = 0; k < 4; ++k) natural[k] = b.dirichlet_x ? k >= 2 : b.bc[k] == PF_BC_NATURAL;
+  auto coarse_cells = [](int n, bool first, bool last) { return last && (n > 1 || first) ? n / 2 : (n + 1) / 2; };
   b.mg_Lv.assign(b.nv, 1);
   std::vector<std::vector<int2>> dims(b.nv);
   int L = 1;
@@ -1324,8 +1327,8 @@ static void mg_layout(Batch& b) {
     int nx = b.hv[v].g.nx, ny = b.hv[v].g.ny;
     dims[v].push_back(make_int2(nx, ny));
     do {
-      nx = coarse_cells(nx, natural_right);
-      ny = coarse_cells(ny, natural_top);
+      nx = coarse_cells(nx, natural[0], natural[1]);
+      ny = coarse_cells(ny, natural[2], natural[3]);
       dims[v].push_back(make_int2(nx, ny));
     } while (std::max(nx, ny) > MG_CMAX);
     b.mg_Lv[v] = (int)dims[v].size();

@@ -49,3 +49,23 @@ def test_phi_with_an_odd_number_of_rows():
         ref, _, _ = api.phi_solve(g, U=1.0, tol=1e-13, precision=api.PF_FP64)
     assert info[0]["status"] == 0 and info[0]["iters"] <= 60
     assert rel_l2(phi.cpu().numpy(), ref.cpu().numpy()) <= 1e-6
+
+
+@pytest.mark.parametrize("nx,ny,bc", [(2000, 40, (D, N, N, N)), (600, 9, (D, N, N, N)), (40, 600, (N, N, D, N)), (300, 2, (D, N, N, N)),
+                                      (3, 300, (N, N, N, D)), (129, 65, (N, D, N, N))])
+def test_multigrid_on_thin_domains_between_natural_sides(nx, ny, bc):
+    """Halved until one cell is left between two natural sides, that direction becomes one line; phi
+    has natural conditions at the bottom and the top of the same grid (and of its transpose)."""
+    from paper_2512_12232_gb300 import api
+    h = 4.0 * ny / nx
+    c = W.Case(-4.0, 4.0, -h, h, nx, ny, np.zeros((0, 3)), 0, bc)
+    with api.mesh_build(c.grid, c.bodies, c.sweeps, c.bc) as g:
+        res = api.psi_solve(g, U=1.0, tol=1e-10, precision=api.PF_MIXED, preconditioner="mg", k_max=400,
+                            raise_on_failure=False)
+        phi, info, _ = api.phi_solve(g, U=1.0, tol=1e-10, precision=api.PF_MIXED, preconditioner="mg", k_max=400,
+                                     raise_on_failure=False)
+    assert res.info[0]["status"] == 0 and res.info[0]["iters"] <= 60
+    assert info[0]["status"] == 0 and info[0]["iters"] <= 60
+    # without bodies both are linear: phi = U x, and psi = U y up to a constant per unfixed side
+    x = np.tile(np.linspace(-4.0, 4.0, nx + 1), ny + 1)
+    assert rel_l2(phi.cpu().numpy(), x) <= 1e-4          # tol 1e-10 and a condition number of up to 1e6
