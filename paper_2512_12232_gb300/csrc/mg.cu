@@ -166,16 +166,19 @@ __device__ void fine_stencil32(const MeshDev& m, const DevVariant& V, long long 
 // (aspect 1.71), a row's diagonal is replaced by half the sum of its magnitudes where omega times
 // that sum reaches 1.9 diagonals: Gershgorin then bounds the eigenvalues by 2, and the cycle stays
 // positive definite.  (256x256 cells of aspect 2 stood at a residual of 2e-4 after 400 iterations;
-// 25 now to 1e-10.)  Other grids keep omega / diagonal.
+// 25 now to 1e-10.)  Other grids keep omega / diagonal, except for the velocity potential: its
+// natural condition on the bodies leaves rows of partial cells, on every level, that pass the same
+// line on grids of any aspect (2000x40 cells of aspect 2/3 with a cylinder: 9e-8 after 300
+// iterations, now 37 to 1e-10; 256x200 cells 148 -> 43, 1024x512 70 -> 62).
 constexpr float MG_STRETCH = 1.9f;
 __device__ __forceinline__ bool stretched(const float* kr) {
   const float e = fabsf(kr[0]) + fabsf(kr[1]) + fabsf(kr[2]), d = -(kr[0] + kr[1] + kr[2]);
   return MG_OMEGA * (e + d) >= MG_STRETCH * d;
 }
-__device__ __forceinline__ float jacobi_factor(const float st[9], bool stretch) {
+__device__ __forceinline__ float jacobi_factor(const float st[9], bool damp) {
   if (!(st[4] > 0.0f)) return 0.0f;
   float d = st[4];
-  if (stretch) {
+  if (damp) {
     float e = 0.0f;
     for (int k = 0; k < 9; ++k) e += fabsf(st[k]);
     if (MG_OMEGA * e >= MG_STRETCH * d) d = 0.5f * e;
@@ -236,7 +239,7 @@ __global__ void k_mg_act(LvArgs c, const uint8_t* act_f, const long long* off_f,
 // Galerkin stencil of coarse node I = sum_{a, b} P(a, I) A_f(a, b) P(b, J) over active
 // fine nodes a, b, in FP32 (the precision the cycle applies it in), and the Jacobi factor.
 __global__ void k_mg_rap(LvArgs c, float* A32c, float* dinvc, MeshDev m, const uint8_t* act_f, const float* A32f,
-                         const long long* off_f, const int2* dims_f, long long nf) {
+                         const long long* off_f, const int2* dims_f, long long nf, bool phi) {
   LvNode q;
   if (!lv_node(c.off, c.dims, c.blkvar, q)) return;
   float acc[9];
@@ -291,11 +294,11 @@ __global__ void k_mg_rap(LvArgs c, float* A32c, float* dinvc, MeshDev m, const u
     }
   }
   for (int k = 0; k < 9; ++k) A32c[k * c.n + q.k] = acc[k];
-  dinvc[q.k] = c.act[q.k] ? jacobi_factor(acc, stretched(V.kr32)) : 0.0f;
+  dinvc[q.k] = c.act[q.k] ? jacobi_factor(acc, phi || stretched(V.kr32)) : 0.0f;
 }
 
 // Jacobi factors of the fine level, at FREE nodes.
-__global__ void k_mg_dinv0(MeshDev m, const int* tile_var, const int2* tile_ij, float* dinv0) {
+__global__ void k_mg_dinv0(MeshDev m, const int* tile_var, const int2* tile_ij, float* dinv0, bool phi) {
   const DevVariant& V = m.var[tile_var[blockIdx.x]];
   const int2 ij = tile_ij[blockIdx.x];
   const int i = ij.x + threadIdx.x, j = ij.y + threadIdx.y;
@@ -305,7 +308,7 @@ __global__ void k_mg_dinv0(MeshDev m, const int* tile_var, const int2* tile_ij, 
   if ((m.tag[n] & KIND_MASK) == K_FREE) {
     float st[9];
     fine_stencil32(m, V, n, i, j, st);
-    d = jacobi_factor(st, stretched(V.kr32));
+    d = jacobi_factor(st, phi || stretched(V.kr32));
   }
   dinv0[n] = d;
 }
@@ -1277,7 +1280,7 @@ void mg_setup(Batch& b) {
   const int L = b.mg_L;
   const MeshDev m = mesh_view(b);
   cudaStream_t s = b.stream;
-  k_mg_dinv0<<<(unsigned)b.T, dim3(TX, TY), 0, s>>>(m, b.tile_var, b.tile_ij, b.mg_dinv0);
+  k_mg_dinv0<<<(unsigned)b.T, dim3(TX, TY), 0, s>>>(m, b.tile_var, b.tile_ij, b.mg_dinv0, b.dirichlet_x);
   if (b.B > 0) {
     k_mg_body_diag<<<b.B, dim3(TX, TY), 0, s>>>(m, b.d_body_var, b.mg_Abb);
     if (!b.mg_adj_ptr) {   // the lists depend on the topology only: counted once per handle
@@ -1306,7 +1309,8 @@ void mg_setup(Batch& b) {
     k_mg_act<<<(unsigned)M.nblk, 256, 0, s>>>(c, f0 ? nullptr : F.act, f0 ? nullptr : F.d_off,
                                                f0 ? nullptr : F.d_dims, b.d_var, b.tag, M.act);
     k_mg_rap<<<(unsigned)M.nblk, 256, 0, s>>>(c, M.A32, M.dinv, m, f0 ? nullptr : F.act, f0 ? nullptr : F.A32,
-                                               f0 ? nullptr : F.d_off, f0 ? nullptr : F.d_dims, f0 ? 0 : F.n);
+                                               f0 ? nullptr : F.d_off, f0 ? nullptr : F.d_dims, f0 ? 0 : F.n,
+                                               b.dirichlet_x);
   }
   PF_CUDA(cudaGetLastError());
   b.launches += 1 + (b.B > 0 ? 1 : 0) + 2 * (L - 1);

@@ -69,3 +69,17 @@ def test_multigrid_on_thin_domains_between_natural_sides(nx, ny, bc):
     # without bodies both are linear: phi = U x, and psi = U y up to a constant per unfixed side
     x = np.tile(np.linspace(-4.0, 4.0, nx + 1), ny + 1)
     assert rel_l2(phi.cpu().numpy(), x) <= 1e-4          # tol 1e-10 and a condition number of up to 1e6
+
+
+@pytest.mark.parametrize("nx,ny,asp", [(2000, 40, 2 / 3), (200, 160, 1.6), (256, 200, 25 / 16), (257, 129, 1.0)])
+def test_phi_around_a_body(nx, ny, asp):
+    """The natural condition on a body leaves rows of partial cells whose Jacobi factor is damped."""
+    from paper_2512_12232_gb300 import api
+    h = 4.0 * ny / nx / asp
+    c = W.Case(-4.0, 4.0, -h, h, nx, ny, np.array([[0.1 * h, 0.07 * h, 0.35 * h]]), 4, (D, D, D, D))
+    with api.mesh_build(c.grid, c.bodies, c.sweeps, c.bc) as g:
+        phi, info, _ = api.phi_solve(g, U=1.0, tol=1e-10, precision=api.PF_MIXED, preconditioner="mg", k_max=300,
+                                     raise_on_failure=False)
+        ref, _, _ = api.phi_solve(g, U=1.0, tol=1e-12, precision=api.PF_FP64)
+    assert info[0]["status"] == 0 and info[0]["iters"] <= 60
+    assert rel_l2(phi.cpu().numpy(), ref.cpu().numpy()) <= 1e-4      # tol 1e-10 and a condition number of up to 1e6
